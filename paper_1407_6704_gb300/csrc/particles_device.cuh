@@ -1924,8 +1924,10 @@ __global__ void k_aos_to_soa(long long np, int d, const double* __restrict__ aos
   for (int k = 0; k < d; ++k) soa[k * np + p] = aos[p * d + k];
 }
 
-__global__ void k_interleave(long long np, int d, const double* __restrict__ soa,
-                             const unsigned* __restrict__ pid, double* __restrict__ aos,
+// Storage order -> user order of X and U together (one launch and one read of pid).
+__global__ void k_interleave(long long np, int d, const double* __restrict__ X,
+                             const double* __restrict__ U, const unsigned* __restrict__ pid,
+                             double* __restrict__ x_aos, double* __restrict__ u_aos,
                              unsigned* __restrict__ err) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= np) return;
@@ -1934,7 +1936,10 @@ __global__ void k_interleave(long long np, int d, const double* __restrict__ soa
     atomicOr(err, ERR_INDEX);
     return;
   }
-  for (int k = 0; k < d; ++k) aos[(long long)p * d + k] = soa[k * np + i];
+  for (int k = 0; k < d; ++k) {
+    if (x_aos) x_aos[(long long)p * d + k] = X[k * np + i];
+    if (u_aos) u_aos[(long long)p * d + k] = U[k * np + i];
+  }
 }
 
 

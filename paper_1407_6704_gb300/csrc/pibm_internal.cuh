@@ -486,9 +486,10 @@ cudaError_t launch_collide_tiles(const State& s, cudaStream_t st, int which, int
 // Write plane a of the stored buffer f[cur] from FP64 values src (already
 // un-streamed by the host), or from the rest value w_a when src is NULL.
 cudaError_t launch_store_plane(const State& s, int a, const double* src, cudaStream_t st);
-// Post-stream populations / moments of the current state into FP64 arrays.
-cudaError_t launch_read_pop_plane(const State& s, int a, double* dst, cudaStream_t st);
-cudaError_t launch_read_moment(const State& s, int comp, double* dst, cudaStream_t st);
+// The post-stream state in FP64: rho [ncell], j [d][ncell] (either may be NULL) and
+// the population planes [a0, a1) into pop [a1 - a0][ncell] (unused when a0 == a1).
+cudaError_t launch_read_state(const State& s, double* rho, double* j, double* pop, int a0, int a1,
+                              cudaStream_t st);
 
 // Particles: binning (counting sort into lattice-cell bins) and the coupled
 // particle kernel (interpolate, contacts, update, spread).
@@ -499,8 +500,9 @@ cudaError_t launch_contacts(const State& s, cudaStream_t st, int* nkernels);
 cudaError_t launch_couple(const State& s, cudaStream_t st, int* nkernels,
                           cudaEvent_t before_particles = nullptr);
 cudaError_t launch_particle_forces(const State& s, double* f_fpi, double* f_c, cudaStream_t st);
-// X or U of the current state (SoA by storage position) into aos[user index][d].
-cudaError_t launch_interleave(const State& s, const double* soa, double* aos, cudaStream_t st);
+// X and U of the current state (SoA by storage position) into aos[user index][d]
+// (either may be NULL).
+cudaError_t launch_interleave(const State& s, double* x_aos, double* u_aos, cudaStream_t st);
 // aos [np][d] -> soa [d][np], both device memory.
 cudaError_t launch_aos_to_soa(long long np, int d, const double* aos, double* soa,
                               cudaStream_t st);
