@@ -46,7 +46,7 @@ constexpr size_t ALIGN = 256;
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Layout {
-  size_t f, F, mom, red, err, out, X, U, rad, mass, Ap, buoy, gw, cf, pid, rl, jl, Fs, ti, tw, nb, nbn, xs0, xr, cr, xs, cs, g, Fc, Fcf, key, rank, perm, bin,
+  size_t f, F, mom, red, err, out, X, U, rad, mass, Ap, buoy, gw, cf, pid, rl, jl, Fs, tf, tr, nb, nbn, xs0, xr, cr, xs, cs, g, Fc, Fcf, key, rank, perm, bin,
       bsum, tflag, tbusy, tfree, tblk, tn;
   size_t total;
 };
@@ -181,8 +181,8 @@ Layout layout(const pibm_config* c) {
   L.rl = take(sub ? sizeof(double) * np : 0);
   L.jl = take(sub ? sizeof(double) * d * np : 0);
   L.Fs = take(sub ? sizeof(double) * d * np : 0);
-  L.ti = take(c->deterministic ? sizeof(int) * 12 * np : 0);
-  L.tw = take(c->deterministic ? sizeof(double) * 12 * np : 0);
+  L.tf = take(c->deterministic ? sizeof(int4) * np : 0);
+  L.tr = take(c->deterministic ? fs * TAP_RECORD * np : 0);
   const bool keep = c->rebin_every > 1;
   // contact candidates recorded at a rebuild (kept cell list) or at the first DEM
   // sub-step (sub-cycling)
@@ -519,8 +519,8 @@ int pibm_create(const pibm_config* cfg, void* workspace, size_t workspace_bytes,
   P.rl = (double*)(base + L.rl);
   P.jl = (double*)(base + L.jl);
   P.Fs = (double*)(base + L.Fs);
-  P.ti = (int*)(base + L.ti);
-  P.tw = (double*)(base + L.tw);
+  P.tf = (int4*)(base + L.tf);
+  P.tr = base + L.tr;
   P.nb = (unsigned*)(base + L.nb);
   P.nbn = (int*)(base + L.nbn);
   P.xs0 = cfg->rebin_every > 1 ? (float4*)(base + L.xs0) : nullptr;

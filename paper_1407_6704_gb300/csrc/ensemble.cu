@@ -434,12 +434,15 @@ __global__ void __launch_bounds__(ENS_THREADS, EnsShape<Q, St>::MINB) k_ensemble
         const int x = (int)(c % sA.g.n[0]);
         const long long r = c / sA.g.n[0];
         const int y = (int)(r % sA.g.n[1]), z = (int)(r / sA.g.n[1]);
+        using TD = TileDims<D>;
+        if (!sX.tflag[x / TD::TX + sA.bm.nt[0] * (y / TD::TY + sA.bm.nt[1] * (z / TD::TZ))])
+          return;  // free tiles stay at zero
         if (sX.rebin > 1)
-          spread_gather_at<D, W, R0 + 1, FT>(sA.g, sA.bm, sA.np, sA.ti, sA.tw, sA.Apn, sA.gout,
-                                             sA.start, (FT*)sA.F, x, y, z);
+          spread_gather_at<D, W, R0 + 1, FT>(sA.g, sA.bm, sA.tf, (const FT*)sA.tr, sA.start,
+                                             (FT*)sA.F, x, y, z);
         else
-          spread_gather_at<D, W, R0, FT>(sA.g, sA.bm, sA.np, sA.ti, sA.tw, sA.Apn, sA.gout,
-                                         sA.start, (FT*)sA.F, x, y, z);
+          spread_gather_at<D, W, R0, FT>(sA.g, sA.bm, sA.tf, (const FT*)sA.tr, sA.start,
+                                         (FT*)sA.F, x, y, z);
       });
       if (!sync()) return;
     }

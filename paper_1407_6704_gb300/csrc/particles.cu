@@ -112,7 +112,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
         if (k == 0) k_contacts<D, true, false, 1><<<pb, 256, 0, st>>>(A);
         else k_contacts<D, true, false, 2><<<pb, 256, 0, st>>>(A);
       }
-      k_substep<D><<<pb, 256, 0, st>>>(A, h);
+      k_substep<D, FT><<<pb, 256, 0, st>>>(A, h);
     }
     n += 1 + 2 * s.phy.substeps;
     if (A.spread) {
@@ -122,19 +122,10 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   }
   if (nk) *nk += n;
   if (s.deterministic) {
-    const Geometry& g = s.geo;
-    int bx = g.n[0] <= 32 ? 32 : (g.n[0] <= 64 ? 64 : 128);
-    dim3 blk(bx, 256 / bx, 1);
-    dim3 grd((g.n[0] + blk.x - 1) / blk.x, (g.n[1] + blk.y - 1) / blk.y, g.n[2]);
     constexpr int R0 = W == 2 ? 1 : 2;
-    if (s.phy.rebin > 1)
-      k_spread_gather<D, W, R0 + 1, FT><<<grd, blk, 0, st>>>(g, P.bm, P.np, P.ti, P.tw,
-                                                             P.Ap[1 - s.cur], P.g, P.bin_cnt,
-                                                             (FT*)s.F);
-    else
-      k_spread_gather<D, W, R0, FT><<<grd, blk, 0, st>>>(g, P.bm, P.np, P.ti, P.tw,
-                                                         P.Ap[1 - s.cur], P.g, P.bin_cnt,
-                                                         (FT*)s.F);
+    auto kern = s.phy.rebin > 1 ? k_spread_gather<D, W, R0 + 1, FT> : k_spread_gather<D, W, R0, FT>;
+    kern<<<(unsigned)ntiles, TileDims<D>::TC, 0, st>>>(s.geo, P.bm, P.tbusy, P.tn, P.tf,
+                                                       (const FT*)P.tr, P.bin_cnt, (FT*)s.F);
     if (nk) *nk += 1;
   }
   return cudaGetLastError();

@@ -330,9 +330,9 @@ struct Particles {
   double* rl;     // [np] interpolated rho_l of the step
   double* jl;     // [d][np] interpolated j_l of the step
   double* Fs;     // [d][np] contact force of the current sub-step
-  // ordered spreading (deterministic mode): each particle's spreading taps, by slot
-  int* ti;        // [np][3][4] cell index per axis and node
-  double* tw;     // [np][3][4] weight per axis and node
+  // ordered spreading (deterministic mode), by slot
+  int4* tf;       // [np] first stencil node per axis
+  void* tr;       // [np][TAP_RECORD] stencil weights and A_p g, in the force field's type
   // kept cell list (rebin_every > 1): contact candidates recorded at the rebuild
   float4* xs0;    // [np] in-cell offsets at the last rebuild, by slot
   unsigned* nb;   // [nb_max][np] candidate slots
@@ -360,6 +360,10 @@ struct Particles {
 
 // Tiles per CTA of the tile-list kernels.
 constexpr int TILE_BLOCK = 256;
+
+// Values per particle of the ordered spreading's record: four weights per axis
+// and the amplitude (a fourth is unused).
+constexpr int TAP_RECORD = 16;
 
 struct State {
   Geometry geo;
