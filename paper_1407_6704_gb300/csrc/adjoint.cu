@@ -10,13 +10,14 @@
 // collision (stored populations of the step start, the spread force, the moment
 // field, the particle state of both buffers and the cell list), then runs the
 // adjoint of each step backwards:
-//   1. collision (Eqs. 2, 3, 8) per cell: the adjoint of the post-stream
+//   1. streaming and collision (Eqs. 2, 3, 8) per cell: the pull of the forward
+//      step becomes a pull in the opposite direction (each stored population feeds
+//      exactly one post-stream one); then the adjoint of the post-stream
 //      populations, of the force field, and the tau sensitivity;
 //   2. spreading (Eq. 9) and the particle update (Eqs. 6-7, 13) per particle;
 //   3. contacts (linear spring-dashpot) and interpolation (Eq. 4) per particle,
 //      the latter spreading the adjoint of (rho_l, j_l) into a cell field;
-//   4. streaming: the pull of the forward step becomes a pull in the opposite
-//      direction (each stored population feeds exactly one post-stream one).
+//   4. that field into the adjoint of the post-stream populations.
 #include <math.h>
 
 #include <vector>
@@ -89,133 +90,218 @@ __device__ __forceinline__ void axis_taps_d(double X, int n, int periodic, TapsD
   }
 }
 
-// Source of population a arriving at (x, y, z) by the pull stream; bb when the
-// link crosses a wall (the bounced population of the cell itself arrives).
+// Neighbour of (x, y, z) in the direction sgn * e_a, wrapped on periodic axes;
+// false when it lies beyond a wall (the link then bounces back).
 template <int Q>
-__device__ __forceinline__ long long adj_pull_src(const Geometry& g, int x, int y, int z, int a,
-                                                  bool& bb) {
+__device__ __forceinline__ bool adj_neighbour(const Geometry& g, int x, int y, int z, int a,
+                                              int sgn, long long& c) {
   using L = Lattice<Q>;
-  int s[3] = {x - L::e(a, 0), y - L::e(a, 1), z - L::e(a, 2)};
-  bb = false;
+  int t[3] = {x + sgn * L::e(a, 0), y + sgn * L::e(a, 1), z + sgn * L::e(a, 2)};
+  bool in = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     if (L::e(a, k) == 0) continue;
-    if (s[k] < 0) {
-      if (g.periodic[k]) s[k] += g.n[k];
-      else bb = true;
-    } else if (s[k] >= g.n[k]) {
-      if (g.periodic[k]) s[k] -= g.n[k];
-      else bb = true;
+    if (t[k] < 0 || t[k] >= g.n[k]) {
+      if (g.periodic[k]) t[k] = t[k] < 0 ? t[k] + g.n[k] : t[k] - g.n[k];
+      else in = false;
     }
   }
-  return s[0] + (long long)g.n[0] * (s[1] + (long long)g.n[1] * s[2]);
-}
-
-__device__ __forceinline__ void cell_xyz(const Geometry& g, long long c, int& x, int& y, int& z) {
-  x = (int)(c % g.n[0]);
-  const long long r = c / g.n[0];
-  y = (int)(r % g.n[1]);
-  z = (int)(r / g.n[1]);
+  c = t[0] + (long long)g.n[0] * (t[1] + (long long)g.n[1] * t[2]);
+  return in;
 }
 
 constexpr int ADJ_THREADS = 256;
+// Threads per CTA of the cell kernel: small CTAs, so that a few thousand cells
+// already spread over every SM (its FP64 work is the bound at any size).
+constexpr int ADJ_CELLS = 64;
 
-// 1. Collision adjoint per cell. Forward, with T_a = f*_a - (1 - om) f_a:
+// Moments of one value per velocity, weighted: m0 = sum w v, m1 = sum w e v,
+// m2 = sum w e e v (diagonal, then xy, xz, yz). Opposite velocities share their
+// weight, so an even sum and an odd difference per pair carry everything; the two
+// weight classes (axis links, the rest) are summed before they are weighted.
+template <int Q>
+__device__ __forceinline__ void weighted_moments(const double (&v)[Q], double& m0,
+                                                 double (&m1)[3], double (&m2)[6]) {
+  using L = Lattice<Q>;
+  constexpr int D = L::D;
+  constexpr double w1 = L::w(1), w2 = L::w(Q - 1);
+  double ax = 0.0, d0 = 0.0, dd[3] = {0.0, 0.0, 0.0}, od[3] = {0.0, 0.0, 0.0};
+  double off[3] = {0.0, 0.0, 0.0}, pk[3] = {0.0, 0.0, 0.0}, mk[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int a = 1; a < Q; a += 2) {
+    const double p = v[a] + v[a + 1], m = v[a] - v[a + 1];
+    if (a < 2 * D) {  // the link along axis (a - 1) / 2
+      pk[(a - 1) / 2] = p;
+      mk[(a - 1) / 2] = m;
+      ax = a == 1 ? p : ax + p;
+      continue;
+    }
+    const bool first = a == 2 * D + 1;
+    d0 = first ? p : d0 + p;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      if (L::e(a, k) == 0) continue;
+      dd[k] += p;
+      od[k] += L::e(a, k) > 0 ? m : -m;
+    }
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+#pragma unroll
+      for (int l = k + 1; l < D; ++l) {
+        const int s = L::e(a, k) * L::e(a, l);
+        if (s > 0) off[k + l - 1] += p;
+        if (s < 0) off[k + l - 1] -= p;
+      }
+  }
+  m0 = L::w(0) * v[0] + (w1 * ax + w2 * d0);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    m1[k] = k < D ? w1 * mk[k] + w2 * od[k] : 0.0;
+    m2[k] = k < D ? w1 * pk[k] + w2 * dd[k] : 0.0;
+    m2[3 + k] = w2 * off[k];
+  }
+}
+
+// 1. Stream and collision adjoint per cell. Forward, with T_a = f*_a - (1 - om) f_a:
 //   T_a = w_a [om rho (1 + 3 eu + 4.5 eu^2 - 1.5 uu) + cF (3 eF - 3 uF + 9 eu eF)],
 //   u = (j + F/2) / rho, cF = 1 - om/2.
-// Given gb = adjoint of f*, writes fb = adjoint of the post-stream populations
-// (without the interpolation's moment terms), Fb = adjoint of the force, and
-// adds this block's d L / d om to om_part[block].
+// The adjoint gb of f* is pulled from fnext, the adjoint of the post-stream
+// populations of the following step: the stored population (x, a) reaches exactly
+// one of them, (x + e_a, a) when that cell is in the lattice (wrapped on periodic
+// axes), else (x, opp a) by bounce-back. Writes fb = adjoint of this step's
+// post-stream populations (without the interpolation's moment terms), Fb = adjoint
+// of the force, and adds this block's d L / d om to om_part[block].
+// Everything the collision adjoint needs of gb are its weighted moments up to
+// second order, M0 = sum w gb, M1 = sum w e gb, M2 = sum w e e gb:
+//   V  = 3 M1 + 9 M2 u - 3 u M0,         ub = om rho V + cF (9 M2 F - 3 F M0),
+//   jb = ub / rho, Fb = cF V + jb / 2,   rhob = om sum w gb poly - jb.u,
+//   fb = (1 - om) gb + rhob + e.jb.
+// FP64-bound: on a 96^3 D3Q19 lattice the form that summed every term per
+// velocity took 1,996 us with a separate stream pass of 371 us; now 466 us with the pull
+// included (and 48 us for the moment terms, which the stream pass used to add).
 template <int Q>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_collide(Geometry g, double om, double cF,
-                                                             const double* __restrict__ fin,
-                                                             const double* __restrict__ F,
-                                                             const double* __restrict__ gbar,
-                                                             double* __restrict__ fbar,
-                                                             double* __restrict__ Fbar,
-                                                             double* __restrict__ om_part) {
+__global__ void __launch_bounds__(ADJ_CELLS) k_adj_collide(Geometry g, double om, double cF,
+                                                           const double* __restrict__ fin,
+                                                           const double* __restrict__ F,
+                                                           const double* __restrict__ fnext,
+                                                           double* __restrict__ fbar,
+                                                           double* __restrict__ Fbar,
+                                                           double* __restrict__ om_part) {
   using L = Lattice<Q>;
   constexpr int D = L::D;
   constexpr int FS = FieldStride<D>::F;
-  __shared__ double red[ADJ_THREADS];
-  const long long c = blockIdx.x * (long long)ADJ_THREADS + threadIdx.x;
+  static_assert(StoreF64::S == 1, "stored values are f - w");
+  __shared__ double red[ADJ_CELLS / 32];
+  const unsigned cu = blockIdx.x * (unsigned)ADJ_CELLS + threadIdx.x;  // at most 2^26 cells
   double omb = 0.0;
-  if (c < g.ncell) {
-    int x, y, z;
-    cell_xyz(g, c, x, y, z);
+  if (cu < (unsigned)g.ncell) {
+    const long long c = cu;
+    const unsigned n0 = (unsigned)g.n[0], n1 = (unsigned)g.n[1];
+    const unsigned row = cu / n0;
+    const int x = (int)(cu - row * n0);
+    const int z = D == 3 ? (int)(row / n1) : 0;
+    const int y = (int)(row - (unsigned)z * n1);
     const long long P = g.pitch;
     double f[Q], gb[Q];
+    const bool inner = x >= 1 && x <= g.n[0] - 2 && y >= 1 && y <= g.n[1] - 2 &&
+                       (D == 2 || (z >= 1 && z <= g.n[2] - 2));
+    if (inner) {
+      const int s0 = g.n[0], s01 = g.n[0] * g.n[1];
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      bool bb;
-      const long long src = adj_pull_src<Q>(g, x, y, z, a, bb);
-      // the stored value is f - S w (StoreF64 keeps the deviation from rest)
-      f[a] = (bb ? fin[opp(a) * P + c] : fin[a * P + src]) + StoreF64::S * L::w(a);
-      gb[a] = gbar[a * P + c];
+      for (int a = 0; a < Q; ++a) {
+        const int o = L::e(a, 0) + s0 * L::e(a, 1) + s01 * L::e(a, 2);
+        f[a] = fin[a * P + c - o];
+        gb[a] = fnext[a * P + c + o];
+      }
+    } else {
+#pragma unroll
+      for (int a = 0; a < Q; ++a) {
+        long long t;
+        f[a] = adj_neighbour<Q>(g, x, y, z, a, -1, t) ? fin[a * P + t] : fin[opp(a) * P + c];
+        gb[a] = adj_neighbour<Q>(g, x, y, z, a, 1, t) ? fnext[a * P + t] : fnext[opp(a) * P + c];
+      }
     }
     double Fv[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int k = 0; k < D; ++k) Fv[k] = F[FS * c + k];
-    double rho = 0.0, j[3] = {0.0, 0.0, 0.0};
+    // moments of the populations (stored as f - w) and sum gb s
+    double dev = f[0], gs = gb[0] * f[0], j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      rho += f[a];
+    for (int a = 1; a < Q; a += 2) {
+      dev += f[a] + f[a + 1];
+      gs += gb[a] * f[a];
+      gs += gb[a + 1] * f[a + 1];
+      const double m = f[a] - f[a + 1];
 #pragma unroll
-      for (int k = 0; k < D; ++k) j[k] += L::e(a, k) * f[a];
+      for (int k = 0; k < D; ++k)
+        if (L::e(a, k) != 0) j[k] += L::e(a, k) > 0 ? m : -m;
     }
+    const double rho = 1.0 + dev, inv = 1.0 / rho;
+    double M0, M1[3], M2[6];
+    weighted_moments<Q>(gb, M0, M1, M2);
     double u[3] = {0.0, 0.0, 0.0}, uu = 0.0, uF = 0.0;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      u[k] = (j[k] + 0.5 * Fv[k]) / rho;
+      u[k] = (j[k] + 0.5 * Fv[k]) * inv;
       uu += u[k] * u[k];
       uF += u[k] * Fv[k];
     }
-    double rhob = 0.0, ub[3] = {0.0, 0.0, 0.0}, Fb[3] = {0.0, 0.0, 0.0};
+    double M2u[3] = {0.0, 0.0, 0.0}, M2F[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      double eu = 0.0, eF = 0.0;
+    for (int k = 0; k < D; ++k)
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        eu += L::e(a, k) * u[k];
-        eF += L::e(a, k) * Fv[k];
+      for (int l = 0; l < D; ++l) {
+        const double q = k == l ? M2[k] : M2[2 + k + l];
+        M2u[k] += q * u[l];
+        M2F[k] += q * Fv[l];
       }
-      const double poly = 1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * uu;
-      const double guo = 3.0 * eF - 3.0 * uF + 9.0 * eu * eF;
-      const double wg = L::w(a) * gb[a];
-      rhob += wg * om * poly;
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const double e = (double)L::e(a, k);
-        ub[k] += wg * (om * rho * (3.0 * e + 9.0 * eu * e - 3.0 * u[k]) +
-                       cF * (-3.0 * Fv[k] + 9.0 * e * eF));
-        Fb[k] += wg * cF * (3.0 * e - 3.0 * u[k] + 9.0 * eu * e);
-      }
-      omb += gb[a] * (-f[a]) + wg * (rho * poly - 0.5 * guo);
-    }
-    double jb[3] = {0.0, 0.0, 0.0};
+    double M1u = 0.0, M1F = 0.0, uM2u = 0.0, uM2F = 0.0;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      jb[k] = ub[k] / rho;
-      Fb[k] += 0.5 * ub[k] / rho;
-      rhob -= ub[k] * u[k] / rho;
+      M1u += M1[k] * u[k];
+      M1F += M1[k] * Fv[k];
+      uM2u += u[k] * M2u[k];
+      uM2F += u[k] * M2F[k];
     }
+    const double poly1 = 3.0 * M1u + 4.5 * uM2u - 1.5 * uu * M0;  // sum w gb (poly - 1)
+    const double guo = 3.0 * M1F - 3.0 * uF * M0 + 9.0 * uM2F;
+    // sum gb f = gs + M0, whose M0 cancels against that of rho poly
+    omb = dev * M0 - gs + rho * poly1 - 0.5 * guo;
+    const double omrho = om * rho;
+    double jb[3] = {0.0, 0.0, 0.0}, rhob = om * (M0 + poly1);
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      double v = (1.0 - om) * gb[a] + rhob;
-#pragma unroll
-      for (int k = 0; k < D; ++k) v += L::e(a, k) * jb[k];
-      fbar[a * P + c] = v;
+    for (int k = 0; k < D; ++k) {
+      const double V = 3.0 * M1[k] + 9.0 * M2u[k] - 3.0 * u[k] * M0;
+      jb[k] = (omrho * V + cF * (9.0 * M2F[k] - 3.0 * Fv[k] * M0)) * inv;
+      Fbar[FS * c + k] = cF * V + 0.5 * jb[k];
+      rhob -= jb[k] * u[k];
     }
+    const double om1 = 1.0 - om;
+    fbar[c] = om1 * gb[0] + rhob;
 #pragma unroll
-    for (int k = 0; k < D; ++k) Fbar[FS * c + k] = Fb[k];
+    for (int a = 1; a < Q; a += 2) {
+      double ej = 0.0;
+      bool first = true;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        if (L::e(a, k) == 0) continue;
+        const double v = L::e(a, k) > 0 ? jb[k] : -jb[k];
+        ej = first ? v : ej + v;
+        first = false;
+      }
+      fbar[a * P + c] = om1 * gb[a] + (rhob + ej);
+      fbar[(a + 1) * P + c] = om1 * gb[a + 1] + (rhob - ej);
+    }
   }
-  red[threadIdx.x] = omb;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) omb += __shfl_xor_sync(0xffffffffu, omb, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = omb;
   __syncthreads();
-  for (int s = ADJ_THREADS / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < ADJ_CELLS / 32; ++w) omb += red[w];
+    om_part[blockIdx.x] += omb;
   }
-  if (threadIdx.x == 0) om_part[blockIdx.x] += red[0];
 }
 
 struct AdjArgs {
@@ -255,91 +341,162 @@ struct AdjArgs {
   unsigned* err;
 };
 
+// The particle kernels give each particle ROWS = W^(d-1) lanes, one per stencil
+// row of W cells along x, and keep PPB particles per CTA: tens of thousands of
+// particles fill the GPU, and the FP64 taps, row sums and scalar updates each run
+// on full warps. One thread per particle left most SMs with a single warp walking
+// 64 taps one after another: on 20,000 particles of a 96^3 lattice the two kernels
+// took 105 and 352 us, now 79 and 169 us.
+template <int D, int W>
+struct AdjShape {
+  static constexpr int WZ = D == 3 ? W : 1;
+  static constexpr int ROWS = W * WZ;
+  static constexpr int THREADS = 128;
+  static constexpr int PPB = THREADS / ROWS;
+};
+
+template <int D, int W>
+struct AdjTapsShared {
+  TapsD<W> t[AdjShape<D, W>::PPB][D];
+};
+
+// Taps of the CTA's particles, one thread per particle and axis. X by storage
+// position; p[i] is particle i's (np: none).
+template <int D, int W>
+__device__ __forceinline__ void adj_block_taps(const AdjArgs& A, const unsigned* p,
+                                               AdjTapsShared<D, W>& sh) {
+  using S = AdjShape<D, W>;
+  for (int i = threadIdx.x; i < S::PPB * D; i += S::THREADS) {
+    const int q = i % S::PPB, k = i / S::PPB;
+    if (p[q] < (unsigned)A.np)
+      axis_taps_d<W>(A.X[k * A.np + p[q]], A.g.n[k], A.g.periodic[k], sh.t[q][k]);
+  }
+}
+
+// Storage positions of the CTA's particles into p (np when the slot is past the
+// end or its record is out of range).
+template <int D, int W>
+__device__ __forceinline__ void adj_block_particles(const AdjArgs& A, unsigned* p) {
+  using S = AdjShape<D, W>;
+  if (threadIdx.x < S::PPB) {
+    const long long sl = blockIdx.x * (long long)S::PPB + threadIdx.x;
+    unsigned v = (unsigned)A.np;
+    if (sl < A.np) {
+      v = (unsigned)A.cs[sl].w;
+      if (v >= (unsigned)A.np) {
+        atomicOr(A.err, ERR_INDEX);
+        v = (unsigned)A.np;
+      }
+    }
+    p[threadIdx.x] = v;
+  }
+}
+
+// Sum over the ROWS lanes of a particle (a power of two up to 16, aligned).
+template <int ROWS>
+__device__ __forceinline__ double row_sum(double v) {
+#pragma unroll
+  for (int o = ROWS / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // 2. Spreading and particle update adjoint, per slot (implicit drag):
 //   U' = N / den, N = m U + 2 A_p j_l + b G + F_c, den = m + 2 A_p rho_l,
 //   X' = X + U', g = 2 (rho_l U' - j_l), F += A_p g w(X).
 template <int D, int W>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_update(AdjArgs A) {
-  const long long sl = blockIdx.x * (long long)ADJ_THREADS + threadIdx.x;
-  if (sl >= A.np) return;
+__global__ void __launch_bounds__(AdjShape<D, W>::THREADS) k_adj_update(AdjArgs A) {
+  using S = AdjShape<D, W>;
+  __shared__ AdjTapsShared<D, W> sh;
+  __shared__ unsigned sp[S::PPB];
+  __shared__ double sums[S::PPB][1 + 2 * D];  // rho_l - S, sum w Fb, sum dw (Fb.g)
   const long long np = A.np;
   const Geometry& g = A.g;
   constexpr int FS = FieldStride<D>::F;
-  const unsigned p = (unsigned)A.cs[sl].w;
-  if (p >= (unsigned)np) {
-    atomicOr(A.err, ERR_INDEX);
-    return;
+  adj_block_particles<D, W>(A, sp);
+  __syncthreads();
+  adj_block_taps<D, W>(A, sp, sh);
+  __syncthreads();
+  const int q = threadIdx.x / S::ROWS, row = threadIdx.x % S::ROWS;
+  const long long slq = blockIdx.x * (long long)S::PPB + q;
+  double rl = 0.0, gb[3] = {0.0, 0.0, 0.0}, xs[3] = {0.0, 0.0, 0.0};
+  if (sp[q] < (unsigned)np) {
+    const TapsD<W>(&t)[D] = sh.t[q];
+    const int iy = row % W, iz = row / W;
+    double gg[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < D; ++k) gg[k] = A.gin[k * np + slq];
+    const double wy = t[1].w[iy], dwy = t[1].dw[iy];
+    const double wz = D == 3 ? t[D - 1].w[iz] : 1.0, dwz = D == 3 ? t[D - 1].dw[iz] : 0.0;
+    const long long r0 =
+        (long long)g.n[0] * (t[1].idx[iy] + (long long)g.n[1] * (D == 3 ? t[D - 1].idx[iz] : 0));
+    double R = 0.0, G[3] = {0.0, 0.0, 0.0}, H = 0.0;
+#pragma unroll
+    for (int ix = 0; ix < W; ++ix) {
+      const long long c = r0 + t[0].idx[ix];
+      const double w = t[0].w[ix];
+      R += w * A.mom[4 * c];
+      double Fg = 0.0;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const double Fb = A.Fbar[FS * c + k];
+        G[k] += w * Fb;
+        Fg += Fb * gg[k];
+      }
+      H += t[0].dw[ix] * Fg;
+    }
+    const double wyz = wy * wz;
+    double Sg = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      Sg += G[k] * gg[k];
+      gb[k] = wyz * G[k];
+    }
+    rl = wyz * R;
+    xs[0] = wyz * H;
+    xs[1] = dwy * wz * Sg;
+    xs[2] = wy * dwz * Sg;
   }
-  double X[3] = {0.0, 0.0, 0.0}, U[3] = {0.0, 0.0, 0.0}, Un[3] = {0.0, 0.0, 0.0},
-         gg[3] = {0.0, 0.0, 0.0};
+  rl = row_sum<S::ROWS>(rl);
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    X[k] = A.X[k * np + p];
-    U[k] = A.U[k * np + p];
-    Un[k] = A.Un[k * np + sl];
-    gg[k] = A.gin[k * np + sl];
+    gb[k] = row_sum<S::ROWS>(gb[k]);
+    xs[k] = row_sum<S::ROWS>(xs[k]);
   }
-  const double m = A.mass[p], Ap = A.Ap[p], bu = A.buoy[p];
-  TapsD<W> t[3];
+  if (row == 0) {
+    sums[q][0] = rl;
 #pragma unroll
-  for (int k = 0; k < D; ++k) axis_taps_d<W>(X[k], g.n[k], g.periodic[k], t[k]);
-  constexpr int WZ = D == 3 ? W : 1;
-  double rho_l = 0.0, j_l[3] = {0.0, 0.0, 0.0}, gb[3] = {0.0, 0.0, 0.0}, xs[3] = {0.0, 0.0, 0.0};
-  for (int iz = 0; iz < WZ; ++iz) {
-    for (int iy = 0; iy < W; ++iy) {
-      for (int ix = 0; ix < W; ++ix) {
-        const double wz = D == 3 ? t[2].w[iz] : 1.0, dwz = D == 3 ? t[2].dw[iz] : 0.0;
-        const double w = t[0].w[ix] * t[1].w[iy] * wz;
-        const double dw[3] = {t[0].dw[ix] * t[1].w[iy] * wz, t[0].w[ix] * t[1].dw[iy] * wz,
-                              t[0].w[ix] * t[1].w[iy] * dwz};
-        const long long c = t[0].idx[ix] + (long long)g.n[0] *
-                                               (t[1].idx[iy] + (long long)g.n[1] *
-                                                                   (D == 3 ? t[2].idx[iz] : 0));
-        const double* mc = A.mom + 4 * c;
-        rho_l += w * mc[0];
-        double Fg = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          j_l[k] += w * mc[1 + k];
-          const double Fb = A.Fbar[FS * c + k];
-          gb[k] += w * Fb;
-          Fg += Fb * gg[k];
-        }
-#pragma unroll
-        for (int k = 0; k < D; ++k) xs[k] += dw[k] * Fg;
-      }
+    for (int k = 0; k < D; ++k) {
+      sums[q][1 + k] = gb[k];
+      sums[q][1 + D + k] = xs[k];
     }
   }
-  rho_l += StoreF64::S;  // the moment field holds rho - S, as in the forward step
-  double Ubt[3], Nb[3], rlb = 0.0, jlb[3] = {0.0, 0.0, 0.0};
+  __syncthreads();
+  // --- the particle's scalars, one thread each ---
+  if (threadIdx.x >= S::PPB || sp[threadIdx.x] >= (unsigned)np) return;
+  const unsigned p = sp[threadIdx.x];
+  const long long sl = blockIdx.x * (long long)S::PPB + threadIdx.x;
+  const double m = A.mass[p], Ap = A.Ap[p], bu = A.buoy[p];
+  // the moment field holds rho - S, as in the forward step
+  const double rho_l = sums[threadIdx.x][0] + StoreF64::S;
+  const double den = m + 2.0 * Ap * rho_l, iden = 1.0 / den;
+  double rlb = 0.0, denb = 0.0, mb = 0.0, bb = 0.0;
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    gb[k] *= Ap;
-    xs[k] *= Ap;
-    Ubt[k] = A.Ub_in[k * np + sl] + A.Xb_in[k * np + sl] + 2.0 * rho_l * gb[k];
-    rlb += 2.0 * gb[k] * Un[k];
-    jlb[k] = -2.0 * gb[k];
-  }
-  const double den = m + 2.0 * Ap * rho_l;
-  double denb = 0.0, mb = 0.0, bb = 0.0;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    Nb[k] = Ubt[k] / den;
-    denb -= Ubt[k] * Un[k] / den;
-  }
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    A.Ub_tmp[k * np + sl] = m * Nb[k];
-    jlb[k] += 2.0 * Ap * Nb[k];
-    A.Fcb[k * np + sl] = Nb[k];
-    mb += Nb[k] * U[k];
-    bb += Nb[k] * A.ph.gravity[k];
-    A.Xb_tmp[k * np + sl] = A.Xb_in[k * np + sl] + xs[k];
-    A.jlb[k * np + sl] = jlb[k];
+    const double gbk = Ap * sums[threadIdx.x][1 + k], xsk = Ap * sums[threadIdx.x][1 + D + k];
+    const double U = A.U[k * np + p], Un = A.Un[k * np + sl], Xb = A.Xb_in[k * np + sl];
+    const double Ubt = A.Ub_in[k * np + sl] + Xb + 2.0 * rho_l * gbk;
+    const double Nb = Ubt * iden;
+    denb -= Nb * Un;
+    rlb += 2.0 * gbk * Un;
+    A.Ub_tmp[k * np + sl] = m * Nb;
+    A.jlb[k * np + sl] = 2.0 * Ap * Nb - 2.0 * gbk;
+    A.Fcb[k * np + sl] = Nb;
+    mb += Nb * U;
+    bb += Nb * A.ph.gravity[k];
+    A.Xb_tmp[k * np + sl] = Xb + xsk;
   }
   mb += denb;
-  rlb += 2.0 * Ap * denb;
-  A.rlb[sl] = rlb;
+  A.rlb[sl] = rlb + 2.0 * Ap * denb;
   // m = rho_r V, b = m (1 - 1/rho_r) = V (rho_r - 1), V = m - b
   A.mb_tmp[sl] = (m - bu) * (mb + bb);
 }
@@ -351,38 +508,34 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_update(AdjArgs A) {
 // (Fcb_i - Fcb_j). Walls: F_k += -(+/-) ... as in the forward kernel.
 // Interpolation rho_l = sum w rho(c), j_l = sum w j(c): the adjoint moments are
 // spread into rjbar with the same weights, and the weight derivatives add to X.
+// A particle's lanes share the neighbour rows of the contact search, then its
+// stencil rows.
 template <int D, int W>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
-  const long long sl = blockIdx.x * (long long)ADJ_THREADS + threadIdx.x;
-  if (sl >= A.np) return;
+__global__ void __launch_bounds__(AdjShape<D, W>::THREADS) k_adj_contact_interp(AdjArgs A) {
+  using S = AdjShape<D, W>;
+  __shared__ AdjTapsShared<D, W> sh;
+  __shared__ unsigned sp[S::PPB];
+  __shared__ double sums[S::PPB][2 * D + 1];  // X, U and mass adjoints
   const long long np = A.np;
   const Geometry& g = A.g;
   const BinMap& bm = A.bm;
-  const int4 mc = A.cs[sl];
-  const unsigned p = (unsigned)mc.w;
-  if (p >= (unsigned)np) {
-    atomicOr(A.err, ERR_INDEX);
-    return;
-  }
-  double X[3] = {0.0, 0.0, 0.0}, U[3] = {0.0, 0.0, 0.0}, Xb[3] = {0.0, 0.0, 0.0},
-         Ub[3] = {0.0, 0.0, 0.0}, ai[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    X[k] = A.X[k * np + p];
-    U[k] = A.U[k * np + p];
-    Xb[k] = A.Xb_tmp[k * np + sl];
-    Ub[k] = A.Ub_tmp[k * np + sl];
-    ai[k] = A.Fcb[k * np + sl];
-  }
-  const double m = A.mass[p], r = A.rad[p], kn = A.ph.kn, beta = A.ph.beta;
-  double mb = 0.0;
-  const int bc[3] = {mc.x, mc.y, mc.z};
-  for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz) {
-    int cz = bc[2] + oz;
-    if (D == 3 && !lattice_coord(cz, g.n[2], g.periodic[2])) continue;
-    for (int oy = -1; oy <= 1; ++oy) {
-      int cy = bc[1] + oy;
+  adj_block_particles<D, W>(A, sp);
+  __syncthreads();
+  adj_block_taps<D, W>(A, sp, sh);
+  __syncthreads();
+  const int qi = threadIdx.x / S::ROWS, row = threadIdx.x % S::ROWS;
+  const long long slq = blockIdx.x * (long long)S::PPB + qi;
+  const unsigned pq = sp[qi];
+  double Xb[3] = {0.0, 0.0, 0.0}, Ub[3] = {0.0, 0.0, 0.0}, mb = 0.0;
+  if (pq < (unsigned)np) {
+    const int4 mc = A.cs[slq];
+    const int bc[3] = {mc.x, mc.y, mc.z};
+    const double r = A.rad[pq];
+    constexpr int NR = D == 3 ? 9 : 3;  // neighbour rows of three cells along x
+    for (int nr = row; nr < NR; nr += S::ROWS) {
+      int cy = bc[1] + nr % 3 - 1, cz = D == 3 ? bc[2] + nr / 3 - 1 : 0;
       if (!lattice_coord(cy, g.n[1], g.periodic[1])) continue;
+      if (D == 3 && !lattice_coord(cz, g.n[2], g.periodic[2])) continue;
       for (int ox = -1; ox <= 1; ++ox) {
         int cx = bc[0] + ox;
         if (!lattice_coord(cx, g.n[0], g.periodic[0])) continue;
@@ -393,7 +546,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
           continue;
         }
         for (unsigned s2 = lo; s2 < hi; ++s2) {
-          if (s2 == (unsigned)sl) continue;
+          if (s2 == (unsigned)slq) continue;
           const unsigned q = (unsigned)A.cs[s2].w;
           if (q >= (unsigned)np) {
             atomicOr(A.err, ERR_INDEX);
@@ -402,13 +555,16 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
           double s[3] = {0.0, 0.0, 0.0}, d2 = 0.0;
 #pragma unroll
           for (int k = 0; k < D; ++k) {
-            s[k] = min_image(X[k] - A.X[k * np + q], g.n[k], g.periodic[k]);
+            s[k] = min_image(A.X[k * np + pq] - A.X[k * np + q], g.n[k], g.periodic[k]);
             d2 += s[k] * s[k];
           }
+          const double rs = r + A.rad[q];
+          if (d2 > rs * rs * (1.0 + 1e-12)) continue;  // clear of each other: no square root
           const double dist = sqrt(d2);
-          const double delta = r + A.rad[q] - dist;
+          const double delta = rs - dist;
           if (!(delta > 0.0) || !(dist > 0.0)) continue;
-          const double mq = A.mass[q];
+          const double kn = A.ph.kn, beta = A.ph.beta;
+          const double m = A.mass[pq], mq = A.mass[q];
           const double meff = m * mq / (m + mq);
           const double gam = 2.0 * beta * sqrt(meff * kn);
           double n[3] = {0.0, 0.0, 0.0}, dU[3] = {0.0, 0.0, 0.0}, vn = 0.0, an = 0.0;
@@ -416,9 +572,9 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
 #pragma unroll
           for (int k = 0; k < D; ++k) {
             n[k] = s[k] / dist;
-            dU[k] = U[k] - A.U[k * np + q];
+            dU[k] = A.U[k * np + pq] - A.U[k * np + q];
             vn += dU[k] * n[k];
-            av[k] = ai[k] - A.Fcb[k * np + s2];
+            av[k] = A.Fcb[k * np + slq] - A.Fcb[k * np + s2];
             an += av[k] * n[k];
           }
           const double mag = kn * delta - gam * vn;
@@ -433,55 +589,78 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
         }
       }
     }
-  }
-  const double gw = A.gw[p];
+    // interpolation adjoint of this lane's stencil row
+    const TapsD<W>(&t)[D] = sh.t[qi];
+    const int iy = row % W, iz = row / W;
+    const double wy = t[1].w[iy], dwy = t[1].dw[iy];
+    const double wz = D == 3 ? t[D - 1].w[iz] : 1.0, dwz = D == 3 ? t[D - 1].dw[iz] : 0.0;
+    const long long r0 =
+        (long long)g.n[0] * (t[1].idx[iy] + (long long)g.n[1] * (D == 3 ? t[D - 1].idx[iz] : 0));
+    const double rlb = A.rlb[slq], wyz = wy * wz;
+    double jlb[3] = {0.0, 0.0, 0.0}, amp[4] = {rlb * wyz, 0.0, 0.0, 0.0};
 #pragma unroll
-  for (int k = 0; k < D; ++k) {
-    if (g.periodic[k]) continue;
-    // wall at 0: F_k += k_n (r - X_k) - gw U_k; wall at n: F_k -= k_n (r - n + X_k) + gw U_k
-    const bool lo = r - X[k] > 0.0, hi = r - ((double)g.n[k] - X[k]) > 0.0;
-    const int cnt = (lo ? 1 : 0) + (hi ? 1 : 0);
-    Xb[k] -= cnt * kn * ai[k];
-    Ub[k] -= cnt * gw * ai[k];
-    mb -= cnt * ai[k] * U[k] * gw / (2.0 * m);
-  }
-  // interpolation adjoint
-  const double rlb = A.rlb[sl];
-  double jlb[3] = {0.0, 0.0, 0.0};
+    for (int k = 0; k < D; ++k) {
+      jlb[k] = A.jlb[k * np + slq];
+      amp[1 + k] = jlb[k] * wyz;
+    }
+    double V = 0.0, DV = 0.0;
 #pragma unroll
-  for (int k = 0; k < D; ++k) jlb[k] = A.jlb[k * np + sl];
-  TapsD<W> t[3];
+    for (int ix = 0; ix < W; ++ix) {
+      const long long c = r0 + t[0].idx[ix];
+      const double* mcell = A.mom + 4 * c;
+      double val = rlb * mcell[0];
 #pragma unroll
-  for (int k = 0; k < D; ++k) axis_taps_d<W>(X[k], g.n[k], g.periodic[k], t[k]);
-  constexpr int WZ = D == 3 ? W : 1;
-  for (int iz = 0; iz < WZ; ++iz) {
-    for (int iy = 0; iy < W; ++iy) {
-      for (int ix = 0; ix < W; ++ix) {
-        const double wz = D == 3 ? t[2].w[iz] : 1.0, dwz = D == 3 ? t[2].dw[iz] : 0.0;
-        const double w = t[0].w[ix] * t[1].w[iy] * wz;
-        const double dw[3] = {t[0].dw[ix] * t[1].w[iy] * wz, t[0].w[ix] * t[1].dw[iy] * wz,
-                              t[0].w[ix] * t[1].w[iy] * dwz};
-        const long long c = t[0].idx[ix] + (long long)g.n[0] *
-                                               (t[1].idx[iy] + (long long)g.n[1] *
-                                                                   (D == 3 ? t[2].idx[iz] : 0));
-        const double* mcell = A.mom + 4 * c;
-        double val = rlb * mcell[0];
+      for (int k = 0; k < D; ++k) val += jlb[k] * mcell[1 + k];
+      const double w = t[0].w[ix];
+      V += w * val;
+      DV += t[0].dw[ix] * val;
+      if (w * wyz != 0.0) {
 #pragma unroll
-        for (int k = 0; k < D; ++k) val += jlb[k] * mcell[1 + k];
-#pragma unroll
-        for (int k = 0; k < D; ++k) Xb[k] += dw[k] * val;
-        if (w != 0.0) {
-          atomicAdd(A.rjbar + 4 * c, rlb * w);
-#pragma unroll
-          for (int k = 0; k < D; ++k) atomicAdd(A.rjbar + 4 * c + 1 + k, jlb[k] * w);
-        }
+        for (int k = 0; k <= D; ++k) atomicAdd(A.rjbar + 4 * c + k, amp[k] * w);
       }
     }
+    Xb[0] += wyz * DV;
+    Xb[1] += dwy * wz * V;
+    if constexpr (D == 3) Xb[2] += wy * dwz * V;
   }
+  mb = row_sum<S::ROWS>(mb);
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    A.Xb_out[k * np + p] = Xb[k];
-    A.Ub_out[k * np + p] = Ub[k];
+    Xb[k] = row_sum<S::ROWS>(Xb[k]);
+    Ub[k] = row_sum<S::ROWS>(Ub[k]);
+  }
+  if (row == 0) {
+    sums[qi][2 * D] = mb;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      sums[qi][k] = Xb[k];
+      sums[qi][D + k] = Ub[k];
+    }
+  }
+  __syncthreads();
+  // --- walls and the sums, one thread per particle ---
+  if (threadIdx.x >= S::PPB || sp[threadIdx.x] >= (unsigned)np) return;
+  const unsigned p = sp[threadIdx.x];
+  const long long sl = blockIdx.x * (long long)S::PPB + threadIdx.x;
+  const double m = A.mass[p], r = A.rad[p], kn = A.ph.kn, gw = A.gw[p];
+  mb = sums[threadIdx.x][2 * D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const double X = A.X[k * np + p], U = A.U[k * np + p], ai = A.Fcb[k * np + sl];
+    double xb = A.Xb_tmp[k * np + sl] + sums[threadIdx.x][k];
+    double ub = A.Ub_tmp[k * np + sl] + sums[threadIdx.x][D + k];
+    if (!g.periodic[k]) {
+      // wall at 0: F_k += k_n (r - X_k) - gw U_k; wall at n: F_k -= k_n (r - n + X_k) + gw U_k
+      const bool lo = r - X > 0.0, hi = r - ((double)g.n[k] - X) > 0.0;
+      const int cnt = (lo ? 1 : 0) + (hi ? 1 : 0);
+      if (cnt) {
+        xb -= cnt * kn * ai;
+        ub -= cnt * gw * ai;
+        mb -= cnt * ai * U * gw / (2.0 * m);
+      }
+    }
+    A.Xb_out[k * np + p] = xb;
+    A.Ub_out[k * np + p] = ub;
   }
   const unsigned user = A.pid[p];
   if (user >= (unsigned)np) {
@@ -491,47 +670,48 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_contact_interp(AdjArgs A) {
   A.drho[user] += (m - A.buoy[p]) * mb + A.mb_tmp[sl];
 }
 
-// 4. Stream adjoint per cell: the stored population (x, a) of the previous step
-// reaches exactly one post-stream population: (x + e_a, a) when that cell is in
-// the lattice (wrapped on periodic axes), else (x, opp a) by bounce-back. Adds
-// the interpolation's moment adjoint rho_bar + e.j_bar of the receiving cell.
+// 4. The interpolation's moment adjoint: fb_a += rho_bar + e_a.j_bar at the cells a
+// stencil reached (all in busy tiles), clearing the field for the next step.
 template <int Q>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_stream(Geometry g,
-                                                            const double* __restrict__ fbar,
-                                                            const double* __restrict__ rjbar,
-                                                            double* __restrict__ gout) {
+__global__ void __launch_bounds__(256) k_adj_moments(Geometry g, BinMap bm,
+                                                     const int* __restrict__ tbusy,
+                                                     const unsigned* __restrict__ tn,
+                                                     double* __restrict__ rjbar,
+                                                     double* __restrict__ fbar) {
   using L = Lattice<Q>;
   constexpr int D = L::D;
-  const long long c = blockIdx.x * (long long)ADJ_THREADS + threadIdx.x;
-  if (c >= g.ncell) return;
-  int x, y, z;
-  cell_xyz(g, c, x, y, z);
+  using TD = TileDims<D>;
+  constexpr int PER = TD::TC / 256;  // CTAs per tile
+  const unsigned i = blockIdx.x / PER;
+  if (i >= tn[0]) return;
+  const int lin = (int)(blockIdx.x % PER) * 256 + (int)threadIdx.x;
+  const int t = tbusy[i], r = t / bm.nt[0];
+  const int x = (t - r * bm.nt[0]) * TD::TX + lin % TD::TX;
+  const int y = (r % bm.nt[1]) * TD::TY + (lin / TD::TX) % TD::TY;
+  const int z = (r / bm.nt[1]) * TD::TZ + lin / (TD::TX * TD::TY);
+  if (x >= g.n[0] || y >= g.n[1] || z >= g.n[2]) return;
+  const long long c = x + (long long)g.n[0] * (y + (long long)g.n[1] * z);
+  double2* rj = reinterpret_cast<double2*>(rjbar) + 2 * c;
+  const double2 lo = rj[0], hi = rj[1];
+  const double rho = lo.x, j[3] = {lo.y, hi.x, hi.y};
+  if (rho == 0.0 && j[0] == 0.0 && j[1] == 0.0 && j[2] == 0.0) return;
+  rj[0] = make_double2(0.0, 0.0);
+  rj[1] = make_double2(0.0, 0.0);
   const long long P = g.pitch;
+  fbar[c] += rho;
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    int t[3] = {x + L::e(a, 0), y + L::e(a, 1), z + L::e(a, 2)};
-    bool in = true;
+  for (int a = 1; a < Q; a += 2) {
+    double ej = 0.0;
+    bool first = true;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < D; ++k) {
       if (L::e(a, k) == 0) continue;
-      if (t[k] < 0 || t[k] >= g.n[k]) {
-        if (g.periodic[k]) t[k] = t[k] < 0 ? t[k] + g.n[k] : t[k] - g.n[k];
-        else in = false;
-      }
+      const double v = L::e(a, k) > 0 ? j[k] : -j[k];
+      ej = first ? v : ej + v;
+      first = false;
     }
-    long long y_c;
-    int b;
-    if (in) {
-      y_c = t[0] + (long long)g.n[0] * (t[1] + (long long)g.n[1] * t[2]);
-      b = a;
-    } else {
-      y_c = c;
-      b = opp(a);
-    }
-    double v = fbar[b * P + y_c] + rjbar[4 * y_c];
-#pragma unroll
-    for (int k = 0; k < D; ++k) v += L::e(b, k) * rjbar[4 * y_c + 1 + k];
-    gout[a * P + c] = v;
+    fbar[a * P + c] += rho + ej;
+    fbar[(a + 1) * P + c] += rho - ej;
   }
 }
 
@@ -566,6 +746,8 @@ __global__ void k_sum_blocks(long long n, const double* __restrict__ in, double*
   }
   if (threadIdx.x == 0) out[0] = red[0];
 }
+
+unsigned cell_blocks(long long n) { return (unsigned)((n + ADJ_CELLS - 1) / ADJ_CELLS); }
 
 unsigned nblk(long long n) { return (unsigned)((n + ADJ_THREADS - 1) / ADJ_THREADS); }
 
@@ -613,13 +795,18 @@ State rebase_state(const State& s, const void* ws, void* tape) {
   P.bin_cnt = rebase(Q.bin_cnt, a, b);
   P.perm = rebase(Q.perm, a, b);
   P.block_sums = rebase(Q.block_sums, a, b);
+  P.tbusy = rebase(Q.tbusy, a, b);
+  P.tn = rebase(Q.tn, a, b);
   return t;
 }
 
+// The adjoint of one step: fnext (adjoint of the post-stream populations of the
+// step after it) -> fbar (of this step's); rjbar is zero on entry and on return.
 template <int Q, int W>
-cudaError_t adjoint_step(const State& T, AdjArgs A, double* gbar, double* fbar, double* Fbar,
-                         double* om_part, cudaStream_t st) {
+cudaError_t adjoint_step(const State& T, AdjArgs A, const double* fnext, double* fbar,
+                         double* Fbar, double* om_part, cudaStream_t st) {
   constexpr int D = Lattice<Q>::D;
+  using S = AdjShape<D, W>;
   const Geometry& g = T.geo;
   const int cur = T.cur, nxt = 1 - T.cur;
   A.X = T.p.X[cur];
@@ -635,23 +822,22 @@ cudaError_t adjoint_step(const State& T, AdjArgs A, double* gbar, double* fbar, 
   A.cs = T.p.cs[cur];
   A.start = T.p.bin_cnt;
   A.mom = (const double*)T.mom;
-  cudaError_t e = cudaMemsetAsync(A.rjbar, 0, sizeof(double) * 4 * g.pitch, st);
-  if (e != cudaSuccess) return e;
-  k_adj_collide<Q><<<nblk(g.ncell), ADJ_THREADS, 0, st>>>(
-      g, T.phy.omega, T.phy.cF, (const double*)T.f[cur], (const double*)T.F, gbar, fbar, Fbar,
+  k_adj_collide<Q><<<cell_blocks(g.ncell), ADJ_CELLS, 0, st>>>(
+      g, T.phy.omega, T.phy.cF, (const double*)T.f[cur], (const double*)T.F, fnext, fbar, Fbar,
       om_part);
-  const unsigned pb = nblk(A.np);
-  k_adj_update<D, W><<<pb, ADJ_THREADS, 0, st>>>(A);
-  k_adj_contact_interp<D, W><<<pb, ADJ_THREADS, 0, st>>>(A);
-  k_adj_stream<Q><<<nblk(g.ncell), ADJ_THREADS, 0, st>>>(g, fbar, A.rjbar, gbar);
+  const unsigned pb = (unsigned)((A.np + S::PPB - 1) / S::PPB);
+  k_adj_update<D, W><<<pb, S::THREADS, 0, st>>>(A);
+  k_adj_contact_interp<D, W><<<pb, S::THREADS, 0, st>>>(A);
+  k_adj_moments<Q><<<(unsigned)(T.p.ntiles * (TileDims<D>::TC / 256)), 256, 0, st>>>(
+      g, A.bm, T.p.tbusy, T.p.tn, A.rjbar, fbar);
   return cudaGetLastError();
 }
 
 template <int Q>
-cudaError_t adjoint_step_w(const State& T, const AdjArgs& A, double* gbar, double* fbar,
+cudaError_t adjoint_step_w(const State& T, const AdjArgs& A, const double* fnext, double* fbar,
                            double* Fbar, double* om_part, cudaStream_t st) {
-  return T.phy.width == 2 ? adjoint_step<Q, 2>(T, A, gbar, fbar, Fbar, om_part, st)
-                          : adjoint_step<Q, 4>(T, A, gbar, fbar, Fbar, om_part, st);
+  return T.phy.width == 2 ? adjoint_step<Q, 2>(T, A, fnext, fbar, Fbar, om_part, st)
+                          : adjoint_step<Q, 4>(T, A, fnext, fbar, Fbar, om_part, st);
 }
 
 // Device allocations of the gradient run, released together.
@@ -742,11 +928,11 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   if (rc != PIBM_OK || !grads) return rc;
 
   char* tape = al.get<char>(wsb * (size_t)K);
-  double* gbar = al.get<double>(sizeof(double) * q * P);
-  double* fbar = al.get<double>(sizeof(double) * q * P);
+  // adjoint of the post-stream populations: of the step after (io) and of this one
+  double* fb[2] = {al.get<double>(sizeof(double) * q * P), al.get<double>(sizeof(double) * q * P)};
   double* Fbar = al.get<double>(sizeof(double) * FS * P);
   double* rjbar = al.get<double>(sizeof(double) * 4 * P);
-  double* om_part = al.get<double>(sizeof(double) * nblk(s.geo.ncell));
+  double* om_part = al.get<double>(sizeof(double) * cell_blocks(s.geo.ncell));
   double* pb[2][2] = {{al.get<double>(sizeof(double) * d * np), al.get<double>(sizeof(double) * d * np)},
                       {al.get<double>(sizeof(double) * d * np), al.get<double>(sizeof(double) * d * np)}};
   double* Xb_tmp = al.get<double>(sizeof(double) * d * np);
@@ -756,15 +942,16 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   double* jlb = al.get<double>(sizeof(double) * d * np);
   double* mb_tmp = al.get<double>(sizeof(double) * np);
   double* drho_d = al.get<double>(sizeof(double) * np);
-  if (!tape || !gbar || !fbar || !Fbar || !rjbar || !om_part || !pb[0][0] || !pb[0][1] ||
+  if (!tape || !fb[0] || !fb[1] || !Fbar || !rjbar || !om_part || !pb[0][0] || !pb[0][1] ||
       !pb[1][0] || !pb[1][1] || !Xb_tmp || !Ub_tmp || !Fcb || !rlb || !jlb || !mb_tmp || !drho_d)
     return PIBM_ENOMEM;
   // adjoint of the final state: d loss / d U_last = 1 / np
-  int io = 0;  // pb[io] = adjoint of (X, U) of the state being reversed into
-  if (cudaMemsetAsync(gbar, 0, sizeof(double) * q * P, st) != cudaSuccess ||
+  int io = 0;  // pb[io], fb[io] = adjoint of the state being reversed into
+  if (cudaMemsetAsync(fb[io], 0, sizeof(double) * q * P, st) != cudaSuccess ||
+      cudaMemsetAsync(rjbar, 0, sizeof(double) * 4 * P, st) != cudaSuccess ||
       cudaMemsetAsync(pb[io][0], 0, sizeof(double) * d * np, st) != cudaSuccess ||
       cudaMemsetAsync(pb[io][1], 0, sizeof(double) * d * np, st) != cudaSuccess ||
-      cudaMemsetAsync(om_part, 0, sizeof(double) * nblk(s.geo.ncell), st) != cudaSuccess ||
+      cudaMemsetAsync(om_part, 0, sizeof(double) * cell_blocks(s.geo.ncell), st) != cudaSuccess ||
       cudaMemsetAsync(drho_d, 0, sizeof(double) * np, st) != cudaSuccess)
     return PIBM_ECUDA;
   k_adj_seed<<<nblk(np), ADJ_THREADS, 0, st>>>(np, d, pb[io][1]);
@@ -803,14 +990,14 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
       A.Xb_out = pb[1 - io][0];
       A.Ub_out = pb[1 - io][1];
       cudaError_t e = cudaErrorInvalidValue;
-      if (q == 9) e = adjoint_step_w<9>(T, A, gbar, fbar, Fbar, om_part, st);
-      else if (q == 15) e = adjoint_step_w<15>(T, A, gbar, fbar, Fbar, om_part, st);
-      else if (q == 19) e = adjoint_step_w<19>(T, A, gbar, fbar, Fbar, om_part, st);
+      if (q == 9) e = adjoint_step_w<9>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
+      else if (q == 15) e = adjoint_step_w<15>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
+      else if (q == 19) e = adjoint_step_w<19>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
       if (e != cudaSuccess) return PIBM_ECUDA;
       io = 1 - io;
     }
   }
-  k_sum_blocks<<<1, ADJ_THREADS, 0, st>>>(nblk(s.geo.ncell), om_part, scal + 1);
+  k_sum_blocks<<<1, ADJ_THREADS, 0, st>>>(cell_blocks(s.geo.ncell), om_part, scal + 1);
   double omb = 0.0;
   if (cudaMemcpyAsync(&omb, scal + 1, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return PIBM_ECUDA;
