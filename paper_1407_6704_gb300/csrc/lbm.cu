@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(256) k_collide_stream_pair(const typename St::
   take_force<D, FT, R>(F, c0, Fv0);
   take_force<D, FT, R>(F, c0 + 1, Fv1);
   R o0[Q], o1[Q];
-  collide_cell<Q, St>(s[0], Fv0, om, cF, err, o0);
-  collide_cell<Q, St>(s[1], Fv1, om, cF, err, o1);
+  collide_cell_pairwise<Q, St>(s[0], Fv0, om, cF, err, o0);
+  collide_cell_pairwise<Q, St>(s[1], Fv1, om, cF, err, o1);
   unsigned short* ob = reinterpret_cast<unsigned short*>(fout);
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
@@ -346,9 +346,14 @@ __global__ void __launch_bounds__(RED_THREADS) k_sum_partials(const double* __re
   }
 }
 
+// 256 threads per CTA, or 64 where 256 would leave an SM fewer than four CTAs: the
+// cells of a small lattice then spread over every SM (its FP64 collision is bound by
+// the FP64 pipe of the SMs that have work).
 dim3 cell_block(const Geometry& g) {
-  int bx = g.n[0] <= 32 ? 32 : (g.n[0] <= 64 ? 64 : 128);
-  return dim3(bx, 256 / bx, 1);
+  constexpr long long SMS = 152;
+  const int t = g.ncell < 4 * SMS * 256 ? 64 : 256;
+  const int bx = g.n[0] <= 32 ? 32 : (g.n[0] <= 64 || t == 64 ? 64 : 128);
+  return dim3(bx, t / bx, 1);
 }
 
 // Block shape of the fused collide-stream: the tuned one when set, else the default.
