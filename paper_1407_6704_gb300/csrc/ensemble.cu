@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(ENS_THREADS, EnsShape<Q, St>::MINB) k_ensemble
   __shared__ EnsExtra sX;
   __shared__ int s_key;
   __shared__ unsigned s_scan[33];
+  __shared__ CoupleStage<Q, W, St, false> s_stage[ENS_THREADS / 32];
   // [nm] parity, [nm] rebuild phase, [nm] period, [nm] np > 0, [nm + 1] moment items
   extern __shared__ int s_dyn[];
   int* s_cur = s_dyn;
@@ -421,7 +422,8 @@ __global__ void __launch_bounds__(ENS_THREADS, EnsShape<Q, St>::MINB) k_ensemble
       for_tickets(E.bar, __ldg(o + E.nm), [&](long long t) {
         const int pos = item_pos(o, E.nm, t);
         use(__ldg(E.ord + IK_PART * E.nm + pos), k);
-        couple_at<Q, W, St, FT, false, false, P64>(sA, (t - __ldg(o + pos)) * ENS_THREADS + tid);
+        couple_slots<Q, W, St, FT, false, false, P64, 32>(
+            sA, (t - __ldg(o + pos)) * ENS_THREADS + (tid & ~31), s_stage[tid >> 5]);
       });
     }
     if (!sync()) return;

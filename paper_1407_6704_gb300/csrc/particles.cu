@@ -61,6 +61,10 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   constexpr int D = Lattice<Q>::D;
   using T = typename St::T;
   using R = typename St::R;
+  // the particle kernels see the dimension and the arithmetic type only: one
+  // instantiation serves every velocity set and storage type of them
+  constexpr int QC = D == 2 ? 9 : 19;
+  using SC = typename std::conditional<sizeof(R) == 8, StoreF64, StoreF32>::type;
   CoupleArgs A = couple_args(s);
   const long long ntiles = P.nbin / P.bm.tc;
   constexpr int KT = MomentsShape<Q, St>::KT;
@@ -80,28 +84,46 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
         constexpr int TPC = CoupleWindow<D, W>::TPC;
         const long long groups = (P.ntiles + TPC - 1) / TPC;
         const unsigned grid = (unsigned)(groups * TILE_CHUNKS);
-        if (s.phy.p64) k_couple_tiles<Q, W, St, FT, true><<<grid, 256, 0, st>>>(A);
-        else k_couple_tiles<Q, W, St, FT, false><<<grid, 256, 0, st>>>(A);
+        if (s.phy.p64) k_couple_tiles<QC, W, SC, FT, true><<<grid, 256, 0, st>>>(A);
+        else k_couple_tiles<QC, W, SC, FT, false><<<grid, 256, 0, st>>>(A);
         tiled = true;
       }
     }
     // 32- and 16-bit storage: the particle update in FP64 (P64) or FP32
     constexpr bool NARROW = sizeof(R) == 4;
+    // a warp takes 32 particles, or one round of it (8 four-point stencils, 16
+    // two-point ones) where 32 would leave an SM with less than one warp: the gathers
+    // of a particle then wait for no other round. 2D FP64 follows one rule at any
+    // count: an ensemble member equals the same simulation stepped alone bit for bit.
+    constexpr int PPW_FEW = W == 4 ? 8 : 16;
+    const bool few = P.np <= 152 * 32 && (D == 3 || COUPLE_BY_WARP<R>);
+    auto blocks = [&](int ppw) { return blocks_for(P.np, COUPLE_WARPS * ppw); };
+    auto go = [&](auto lag, auto p64) {
+      constexpr bool LAG = decltype(lag)::value, P64 = decltype(p64)::value;
+      if (few)
+        k_couple<QC, W, SC, FT, LAG, P64, PPW_FEW>
+            <<<blocks(PPW_FEW), COUPLE_WARPS * 32, 0, st>>>(A);
+      else
+        k_couple<QC, W, SC, FT, LAG, P64, 32><<<blocks(32), COUPLE_WARPS * 32, 0, st>>>(A);
+    };
+    using Yes = std::true_type;
+    using No = std::false_type;
+    using P64 = std::integral_constant<bool, NARROW>;
     if (tiled) {
     } else if (s.phy.lagrange) {
-      if (NARROW && s.phy.p64) k_couple<Q, W, St, FT, true, NARROW><<<pb, 256, 0, st>>>(A);
-      else k_couple<Q, W, St, FT, true, false><<<pb, 256, 0, st>>>(A);
+      if (NARROW && s.phy.p64) go(Yes{}, P64{});
+      else go(Yes{}, No{});
     } else {
-      if (NARROW && s.phy.p64) k_couple<Q, W, St, FT, false, NARROW><<<pb, 256, 0, st>>>(A);
-      else k_couple<Q, W, St, FT, false, false><<<pb, 256, 0, st>>>(A);
+      if (NARROW && s.phy.p64) go(No{}, P64{});
+      else go(No{}, No{});
     }
     n += 1;
   } else {
     // DEM sub-cycling: interpolate once, S x (contacts, update), then spread
     if (s.phy.lagrange)
-      k_sub_init<Q, 4, St, true><<<pb, 256, 0, st>>>(A);
+      k_sub_init<QC, 4, SC, true><<<pb, 256, 0, st>>>(A);
     else
-      k_sub_init<Q, W, St, false><<<pb, 256, 0, st>>>(A);
+      k_sub_init<QC, W, SC, false><<<pb, 256, 0, st>>>(A);
     const double h = 1.0 / (double)s.phy.substeps;
     // the first sub-step records the contact candidates, the others reuse them
     for (int k = 0; k < s.phy.substeps; ++k) {
@@ -116,7 +138,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     }
     n += 1 + 2 * s.phy.substeps;
     if (A.spread) {
-      k_sub_spread<Q, W, St, FT><<<pb, 256, 0, st>>>(A);
+      k_sub_spread<QC, W, SC, FT><<<pb, 256, 0, st>>>(A);
       n += 1;
     }
   }
