@@ -187,17 +187,6 @@ __global__ void k_store_plane(typename St::T* __restrict__ f, const double* __re
   f[c] = St::store((typename St::R)((src ? src[c] : wa) - shift));
 }
 
-// FP32 -> FP64 on the bit pattern: exact for every value, and free of the conversion
-// that runs at the FP64 pipe's rate. Denormals, infinities and NaN take it.
-__device__ __forceinline__ double widen(float v) {
-  const unsigned b = __float_as_uint(v), mag = b & 0x7fffffffu;
-  if (mag - 0x00800000u < 0x7f000000u)  // normal
-    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
-  if (mag == 0u) return __hiloint2double((int)b, 0);
-  return (double)v;
-}
-__device__ __forceinline__ double widen(double v) { return v; }
-
 // The post-stream state of every cell in FP64, in one pass: rho, j and the
 // population planes [a0, a1) (each output may be left out). A thread owns one cell
 // and pulls every population it needs once; the stores of a plane are coalesced.

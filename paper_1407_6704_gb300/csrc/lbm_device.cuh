@@ -56,19 +56,10 @@ __device__ __forceinline__ bool above_mach(float uu) { return __float_as_uint(uu
 __device__ __forceinline__ bool nonzero_bits(double v) { return __double_as_longlong(v) != 0; }
 __device__ __forceinline__ bool nonzero_bits(float v) { return __float_as_uint(v) != 0u; }
 
-// 1 / rho for the collision. FP64: the hardware's coarse reciprocal (PTX
-// rcp.approx.ftz.f64, about 20 bits) and one third-order step of the series
-// 1 / (1 - e) = 1 + e + e^2 + ..., e = 1 - rho r: three FP64 instructions for a
-// result within a rounding of exact, where the division takes about twice that on
-// a pipe that bounds the kernel. rho is positive and near 1; one that is not raises
-// the health flag beside it.
+// 1 / rho for the collision. rho is positive and near 1; one that is not raises the
+// health flag beside it.
 __device__ __forceinline__ float inverse_density(float rho) { return 1.f / rho; }
-__device__ __forceinline__ double inverse_density(double rho) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(rho));
-  const double e = fma(-rho, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
+__device__ __forceinline__ double inverse_density(double rho) { return rcp_series(rho); }
 
 // w x with a weight that FP32 does not hold (1/3, 1/18, ...): the rounding of the
 // constant is added back, since it would be the same in every step and cell (a gain or

@@ -480,20 +480,6 @@ __device__ __forceinline__ void axis_taps(double X, int n, int periodic, Taps<W,
   }
 }
 
-// 1/d in FP64 from an FP32 seed refined by Newton steps: one step gives about
-// 2^-46 relative error, two reach FP64 rounding.
-template <int STEPS>
-__device__ __forceinline__ double rcp_newton(double d) {
-  double r = (double)__frcp_rn((float)d);
-  if (!isfinite(r)) return 1.0 / d;
-#pragma unroll
-  for (int i = 0; i < STEPS; ++i) {
-    const double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-  }
-  return r;
-}
-
 // Bit tests (integer pipe): not finite, and outside [0, n] for a wall axis.
 __device__ __forceinline__ bool not_finite_bits(double v) {
   return ((unsigned long long)__double_as_longlong(v) & 0x7ff0000000000000ull) ==
@@ -1164,7 +1150,9 @@ __device__ __forceinline__ void spread_amp(const CoupleArgs& A, const Taps<W, TW
 // 2D, about one sector per clock and SM). The taps pass through shared memory, which
 // also frees their registers for the update. 2D, 500,000 particles: 6.0 M load and
 // 3.3 M atomic sectors, 55.3 us alone with the FP64 pipe 71 % active (the update);
-// 3D, 90,000 particles with the Lagrange interpolant: 56.7 -> 49.0 us.
+// 3D, 90,000 particles with the Lagrange interpolant: 56.7 -> 49.0 us. With the
+// update's conversions on the bits (42 FP64 instructions per particle -> 27) the 2D
+// kernel takes 48.5 us.
 template <int D, int WI, typename R>
 struct TapStage {
   static constexpr int DY = D == 3 ? 3 : 2;
@@ -1285,7 +1273,7 @@ __device__ __forceinline__ double advance_axis(double x, int n, int periodic, bo
     else if (x >= N) x -= N;
     if (!(x >= 0.0 && x < N)) x = x - N * floor(x / N);  // |U| > N: not physical
     if (!(x >= 0.0 && x < N)) x = 0.0;
-  } else if (outside_bits(x, (double)n)) {
+  } else if (outside_bits(x, from_index(n))) {
     esc = true;
   }
   return x;
@@ -1350,29 +1338,35 @@ __device__ __forceinline__ void advance_particle(const CoupleArgs& A, long long 
   double Un[3];
   bool bad = false, esc = false;
   if constexpr (sizeof(R) == 8 || P64) {
-    const double mi = A.mass[p], Ap = A.Ap[p], bu = A.buoy[p];
-    const double rho_l = (double)St::S + rs;
-    double Ub[3];
+    // every FP64 operation is written out, so that each caller rounds alike
+    const double mi = A.mass[p], bu = A.buoy[p], Ap2 = twice(A.Ap[p]);
+    const double rho_l = (double)St::S + widen(rs);
+    double jl[3], Ub[3];
+#pragma unroll
+    for (int k = 0; k < D; ++k) jl[k] = widen(js[k]);
     if (A.ph.implicit_drag) {
-      const double inv = rcp_newton<2>(mi + 2.0 * Ap * rho_l);
+      const double den = fma(Ap2, rho_l, mi);
+      double inv = rcp_series(den);
+      if (not_finite_bits(inv)) inv = 1.0 / den;
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        Un[k] = (mi * U[k] + 2.0 * Ap * js[k] + bu * A.ph.gravity[k] + Fc[k]) * inv;
+        Un[k] = fma(mi, U[k], fma(Ap2, jl[k], fma(bu, A.ph.gravity[k], (double)Fc[k]))) * inv;
         Ub[k] = Un[k];
       }
     } else {
       const double invm = 1.0 / mi;
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        Un[k] = U[k] + (bu * A.ph.gravity[k] + Fc[k] - Ap * 2.0 * (rho_l * U[k] - js[k])) * invm;
+        const double f = fma(-Ap2, fma(rho_l, U[k], -jl[k]), fma(bu, A.ph.gravity[k], (double)Fc[k]));
+        Un[k] = fma(f, invm, U[k]);
         Ub[k] = U[k];
       }
     }
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      const double gg = 2.0 * (rho_l * Ub[k] - js[k]);
-      amp[k] = (FT)(Ap * gg);
-      A.gout[k * np + sl] = gg;
+      const double v = fma(rho_l, Ub[k], -jl[k]);  // g / 2
+      amp[k] = narrow_to<FT>(Ap2 * v);
+      A.gout[k * np + sl] = twice(v);
     }
   } else {
     const float4 cc = A.cf[p];  // mass, A_p, buoy, radius
@@ -1414,15 +1408,18 @@ __device__ __forceinline__ void advance_particle(const CoupleArgs& A, long long 
     A.Xn[k * np + sl] = xn;
     A.Un[k * np + sl] = Un[k];
     if (A.keep_cells) {
+      const double o = xn - from_index(cell[k]);  // offset from the cell's lower face
       if constexpr (sizeof(R) == 8) {
-        // distance from the cell centre, minimum image on periodic axes
-        const double dc = min_image(xn - ((double)cell[k] + 0.5), g.n[k], g.periodic[k]);
-        far |= !(fabs(dc) <= 0.5 + A.ph.skin);
-        off[k] = (float)(dc + 0.5);
+        // distance from the cell centre, minimum image on periodic axes; positive
+        // values compare like their bit patterns (a NaN counts as far)
+        const double dc = min_image(o - 0.5, g.n[k], g.periodic[k]);
+        far |= ((unsigned long long)__double_as_longlong(dc) & 0x7fffffffffffffffull) >
+               (unsigned long long)__double_as_longlong(0.5 + A.ph.skin);
+        off[k] = g.periodic[k] ? (float)(dc + 0.5) : narrow(o);
       } else {
-        // the same from the offset to the cell's lower face, tested in FP32 (the
-        // rounding moves the bound by about 1e-7 of a cell)
-        off[k] = (float)min_image(xn - (double)cell[k], g.n[k], g.periodic[k]);
+        // the same from the offset, tested in FP32 (the rounding moves the bound by
+        // about 1e-7 of a cell)
+        off[k] = narrow(min_image(o, g.n[k], g.periodic[k]));
         far |= !(fabsf(off[k] - 0.5f) <= 0.5f + A.ph.skinf);
       }
     }
@@ -1661,6 +1658,9 @@ __global__ void __launch_bounds__(COUPLE_WARPS * 32,
 //      sums are exact (independent of their order);
 //   4. every window node with a non-zero force is added to the force field by
 //      one vector atomic, converted back to FP32.
+// Bound by shared-memory wavefronts (59 % busy at 24 warps per SM), next by the FP64
+// pipe of the update. Component-wise force planes and the update's conversions on the
+// bits took it from 1,396 to 1,197 us on the 256^3 workload.
 // The last chunk of a group takes every remaining particle; beyond 256 of them,
 // or if the box exceeds the window (a 2D group that wraps to the next tile row),
 // the CTA falls back to the direct path.
@@ -1685,6 +1685,7 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
   constexpr int D = Lattice<Q>::D;
   using Win = CoupleWindow<D, W>;
   static_assert(sizeof(R) == 4 && sizeof(FT) == 4, "FP32 arithmetic");
+  // the moment window, reused for the force window in fixed point
   __shared__ float4 win[Win::VMAX];
   __shared__ int box[6];
   __shared__ float amp_bound[8][3];  // per warp and component: sum of |A_p g_k| w_max
@@ -1871,8 +1872,11 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
     inv_scale[k] = 1.f / scale[k];  // exact: a power of two
   }
   // --- 3. A_p g w into the window (Eq. 9) ---
-  int4* wi = reinterpret_cast<int4*>(win);
-  for (int v = threadIdx.x; v < V; v += blockDim.x) wi[v] = make_int4(0, 0, 0, 0);
+  // component by component (wi[k * V + cell]): 32 neighbouring cells of a component
+  // lie in 32 banks; side by side in a 16-byte cell the adds of a component met in 8
+  // banks and took 6.8 wavefronts each
+  int* wi = reinterpret_cast<int*>(win);
+  for (int v = threadIdx.x; v < D * V; v += blockDim.x) wi[v] = 0;
   __syncthreads();
   if (act) {
 #pragma unroll 1
@@ -1892,9 +1896,9 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
         for (int ix = 0; ix < W; ++ix) {
           const FT wt = (FT)tx.w[ix] * wyz;
           if (wt == FT(0)) continue;
-          int* c = reinterpret_cast<int*>(wi + row + ix);
 #pragma unroll
-          for (int k = 0; k < D; ++k) atomicAdd(c + k, __float2int_rn(amp[k] * wt * scale[k]));
+          for (int k = 0; k < D; ++k)
+            atomicAdd(wi + k * V + row + ix, __float2int_rn(amp[k] * wt * scale[k]));
         }
       }
     }
@@ -1902,7 +1906,7 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
   __syncthreads();
   // --- 4. the window's force into the force field ---
   for (int v = threadIdx.x; v < V; v += blockDim.x) {
-    const int4 q = wi[v];
+    const int4 q = make_int4(wi[v], wi[V + v], D == 3 ? wi[2 * V + v] : 0, 0);
     if (q.x == 0 && q.y == 0 && (D == 2 || q.z == 0)) continue;
     int cx = bx + v % wx, cy = by + (v / wx) % wy, cz = bz + v / (wx * wy);
     if (!(lattice_coord(cx, g.n[0], g.periodic[0]) && lattice_coord(cy, g.n[1], g.periodic[1]) &&

@@ -114,6 +114,68 @@ struct StoreBF16 {
   }
 };
 
+// ---------------------------------------------------------------------------
+// FP64 values without the FP64 pipe. It issues one warp instruction in 16 cycles
+// here, a conversion to or from FP64 as much as an addition, and it bounds the
+// FP64 kernels and most of the particle update; the same on the bit pattern is a
+// handful of integer instructions. Results are those of the plain operations for
+// every value (the rare ones take them).
+// ---------------------------------------------------------------------------
+// FP32 -> FP64, exact.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  if (mag == 0u) return __hiloint2double((int)b, 0);
+  return (double)v;
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// FP64 -> FP32, round to nearest even.
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned mag = hi & 0x7fffffffu;
+  if (mag - 0x38100000u < 0x0fe00000u) {  // the result is normal (or rounds up to infinity)
+    unsigned u = ((mag - 0x38000000u) << 3) | (lo >> 29);
+    u += ((lo & 0x1fffffffu) + (u & 1u) > 0x10000000u) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | u);
+  }
+  if ((mag | lo) == 0u) return __uint_as_float(hi);
+  return (float)v;
+}
+template <typename T>
+__device__ __forceinline__ T narrow_to(double v) {
+  if constexpr (sizeof(T) == 4) return narrow(v);
+  else return v;
+}
+
+// 2 v.
+__device__ __forceinline__ double twice(double v) {
+  const int hi = __double2hiint(v);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 1u < 0x7fdu) return __hiloint2double(hi + 0x00100000, __double2loint(v));
+  return v + v;
+}
+
+// A non-negative integer as FP64.
+__device__ __forceinline__ double from_index(int c) {
+  if (c == 0) return 0.0;
+  const int n = 31 - __clz(c);
+  const unsigned long long m = (unsigned long long)(unsigned)c << (52 - n);
+  return __longlong_as_double((long long)(((unsigned long long)(1022 + n) << 52) + m));
+}
+
+// 1 / d in FP64: the hardware's coarse reciprocal (PTX rcp.approx.ftz.f64, about 20
+// bits) and one third-order step of the series 1 / (1 - e) = 1 + e + e^2 + ...,
+// e = 1 - d r: three FP64 instructions for a result within a rounding of exact, about
+// half of what the division takes.
+__device__ __forceinline__ double rcp_series(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // L2 eviction priorities for single accesses (PTX createpolicy and the
 // .L2::cache_hint qualifier): a policy marks the lines an access touches to be
 // evicted first or last.
