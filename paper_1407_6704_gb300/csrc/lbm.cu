@@ -218,15 +218,18 @@ __global__ void __launch_bounds__(256) k_read_state(const typename St::T* __rest
                      (D == 2 || (z >= 1 && z <= g.n[2] - 2));
   const int s0 = g.n[0], s01 = g.n[0] * g.n[1];
   T v[Q];
+  if (inner) {
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    if (!mom && (a < a0 || a >= a1)) continue;
-    if (inner) {
+    for (int a = 0; a < Q; ++a) {
+      if (!mom && (a < a0 || a >= a1)) continue;
       v[a] = fin[a * g.pitch + ((int)c - (L::e(a, 0) + s0 * L::e(a, 1) + s01 * L::e(a, 2)))];
-    } else {
-      bool bb;
-      const long long src = pull_src<Q>(g, x, y, z, a, bb);
-      v[a] = bb ? fin[opp(a) * g.pitch + c] : fin[a * g.pitch + src];
+    }
+  } else {
+    const PullAxes ax = pull_axes<D>(g, x, y, z);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      if (!mom && (a < a0 || a >= a1)) continue;
+      v[a] = fin[pull_element<Q>(ax, g.pitch, (int)c, a)];
     }
   }
   if (mom) {

@@ -311,12 +311,9 @@ __device__ __forceinline__ void pull_cell(const typename St::T* __restrict__ fin
       fa += P;
     }
   } else {
+    const PullAxes ax = pull_axes<D>(g, x, y, z);
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      bool bb;
-      long long src = pull_src<Q>(g, x, y, z, a, bb);
-      s[a] = St::load(ld(bb ? fin + (opp(a) * P + c) : fin + (a * P + src)));
-    }
+    for (int a = 0; a < Q; ++a) s[a] = St::load(ld(fin + pull_element<Q>(ax, P, (int)c, a)));
   }
 }
 

@@ -67,10 +67,19 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   using SC = typename std::conditional<sizeof(R) == 8, StoreF64, StoreF32>::type;
   CoupleArgs A = couple_args(s);
   const long long ntiles = P.nbin / P.bm.tc;
-  constexpr int KT = MomentsShape<Q, St>::KT;
   const unsigned pb = blocks_for(P.np, 256);
-  k_moments<Q, St><<<(unsigned)((ntiles + KT - 1) / KT), 256, 0, st>>>(
-      s.geo, P.bm, P.tbusy, P.tn, (const T*)s.f[s.cur], (R*)s.mom);
+  auto moments = [&](auto threads) {
+    constexpr int TH = decltype(threads)::value;
+    using Sh = MomentsShape<Q, St, TH>;
+    k_moments<Q, St, TH>
+        <<<(unsigned)((ntiles + Sh::KT - 1) / Sh::KT * Sh::PARTS), TH, 0, st>>>(
+            s.geo, P.bm, P.tbusy, P.tn, (const T*)s.f[s.cur], (R*)s.mom);
+  };
+  // small CTAs where the large ones would leave an SM fewer than four
+  if (s.geo.ncell < 4 * 152 * MomentsShape<Q, St>::CELLS)
+    moments(std::integral_constant<int, 64>{});
+  else
+    moments(std::integral_constant<int, 256>{});
   if (before_particles) {
     const cudaError_t e = cudaStreamWaitEvent(st, before_particles, 0);
     if (e != cudaSuccess) return e;

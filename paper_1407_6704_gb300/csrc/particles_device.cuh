@@ -496,27 +496,10 @@ __device__ __forceinline__ bool outside_bits(double v, double n) {
 template <int Q, class St>
 __device__ __forceinline__ void pull_load(const typename St::T* __restrict__ f, const Geometry& g,
                                           int x, int y, int z, typename St::T (&v)[Q]) {
-  using L = Lattice<Q>;
-  const long long c = x + (long long)g.n[0] * (y + (long long)g.n[1] * z);
+  const int c = x + g.n[0] * (y + g.n[1] * z);
+  const PullAxes ax = pull_axes<Lattice<Q>::D>(g, x, y, z);
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    int s0 = x - L::e(a, 0), s1 = y - L::e(a, 1), s2 = z - L::e(a, 2);
-    bool bb = false;
-    if (L::e(a, 0) != 0) {
-      if (s0 < 0) { if (g.periodic[0]) s0 += g.n[0]; else bb = true; }
-      else if (s0 >= g.n[0]) { if (g.periodic[0]) s0 -= g.n[0]; else bb = true; }
-    }
-    if (L::e(a, 1) != 0) {
-      if (s1 < 0) { if (g.periodic[1]) s1 += g.n[1]; else bb = true; }
-      else if (s1 >= g.n[1]) { if (g.periodic[1]) s1 -= g.n[1]; else bb = true; }
-    }
-    if (L::e(a, 2) != 0) {
-      if (s2 < 0) { if (g.periodic[2]) s2 += g.n[2]; else bb = true; }
-      else if (s2 >= g.n[2]) { if (g.periodic[2]) s2 -= g.n[2]; else bb = true; }
-    }
-    const long long src = s0 + (long long)g.n[0] * (s1 + (long long)g.n[1] * s2);
-    v[a] = bb ? f[opp(a) * g.pitch + c] : f[a * g.pitch + src];
-  }
+  for (int a = 0; a < Q; ++a) v[a] = f[pull_element<Q>(ax, g.pitch, c, a)];
 }
 
 // Zeroth and first moments of pulled values: sum of the stored values (rho - S)
@@ -864,13 +847,17 @@ __global__ void __launch_bounds__(256, D == 3 ? (HS ? 4 : 3) : 1) k_contacts(Cou
 
 // Shape of the moment kernel: cells per thread (as many loads in flight as the
 // registers allow) and tiles per CTA of 256 threads.
-template <int Q, class St>
+// THREADS: 256, or 64 on a small lattice, whose few tiles then spread over every SM (a
+// tile is at least 256 cells, so such a CTA takes part of one).
+template <int Q, class St, int THREADS = 256>
 struct MomentsShape {
   static constexpr int D = Lattice<Q>::D;
   static constexpr int TC = TileDims<D>::TC;
-  static constexpr int CPT = (D == 3 || sizeof(typename St::T) == 8) ? 2 : 4;
-  static constexpr int MINB = sizeof(typename St::T) == 8 ? 2 : 4;  // CTAs per SM
-  static constexpr int KT = CPT * 256 / TC;
+  static constexpr int CPT = THREADS < 256 ? 1 : (D == 3 || sizeof(typename St::T) == 8) ? 2 : 4;
+  static constexpr int MINB = THREADS < 256 ? 1 : sizeof(typename St::T) == 8 ? 2 : 4;  // CTAs per SM
+  static constexpr int CELLS = CPT * THREADS;                   // cells per CTA
+  static constexpr int KT = CELLS < TC ? 1 : CELLS / TC;        // tiles per CTA
+  static constexpr int PARTS = CELLS < TC ? TC / CELLS : 1;     // CTAs per tile
 };
 
 // Post-stream moments of every cell of the busy tiles (k_tile_lists), KT tiles
@@ -880,14 +867,14 @@ struct MomentsShape {
 // wrap) reads its sources at fixed 32-bit offsets; only cells on the lattice
 // faces take the general path. Cells of free tiles are left untouched; no
 // stencil reads them.
-// (one CTA of 256 threads per group vb of KT busy tiles)
-template <int Q, class St>
+// (one CTA of THREADS threads per group vb of KT busy tiles, or per part of a tile)
+template <int Q, class St, int THREADS = 256>
 __device__ __forceinline__ void moments_block(const Geometry& g, const BinMap& bm,
                                               const int* __restrict__ tbusy,
                                               const unsigned* __restrict__ tn,
                                               const typename St::T* __restrict__ f,
                                               typename St::R* __restrict__ mom, int vb) {
-  using Sh = MomentsShape<Q, St>;
+  using Sh = MomentsShape<Q, St, THREADS>;
   using L = Lattice<Q>;
   using T = typename St::T;
   using R = typename St::R;
@@ -896,7 +883,8 @@ __device__ __forceinline__ void moments_block(const Geometry& g, const BinMap& b
   __shared__ int busy[Sh::KT];
   __shared__ int corner[Sh::KT][3];  // first cell of each tile
   const int nbusy = (int)tn[0];
-  const int i0 = vb * Sh::KT;
+  const int i0 = vb / Sh::PARTS * Sh::KT;
+  const int part = vb % Sh::PARTS;
   if (i0 >= nbusy) return;  // the list is shorter than the grid
   __syncthreads();  // busy and corner may still be read for the CTA's previous group
   if (threadIdx.x < Sh::KT) {
@@ -915,7 +903,7 @@ __device__ __forceinline__ void moments_block(const Geometry& g, const BinMap& b
   bool on[Sh::CPT];
 #pragma unroll
   for (int c = 0; c < Sh::CPT; ++c) {
-    const int lin = c * 256 + (int)threadIdx.x;
+    const int lin = part * Sh::CELLS + c * THREADS + (int)threadIdx.x;
     const int k = lin / TD::TC, i = lin % TD::TC;
     const int x = corner[k][0] + i % TD::TX;
     const int y = corner[k][1] + (i / TD::TX) % TD::TY;
@@ -945,13 +933,13 @@ __device__ __forceinline__ void moments_block(const Geometry& g, const BinMap& b
   }
 }
 
-template <int Q, class St>
-__global__ void __launch_bounds__(256, MomentsShape<Q, St>::MINB) k_moments(Geometry g, BinMap bm,
+template <int Q, class St, int THREADS>
+__global__ void __launch_bounds__(THREADS, MomentsShape<Q, St, THREADS>::MINB) k_moments(Geometry g, BinMap bm,
                                                  const int* __restrict__ tbusy,
                                                  const unsigned* __restrict__ tn,
                                                  const typename St::T* __restrict__ f,
                                                  typename St::R* __restrict__ mom) {
-  moments_block<Q, St>(g, bm, tbusy, tn, f, mom, blockIdx.x);
+  moments_block<Q, St, THREADS>(g, bm, tbusy, tn, f, mom, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
