@@ -154,9 +154,23 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   if (nk) *nk += n;
   if (s.deterministic) {
     constexpr int R0 = W == 2 ? 1 : 2;
-    auto kern = s.phy.rebin > 1 ? k_spread_gather<D, W, R0 + 1, FT> : k_spread_gather<D, W, R0, FT>;
-    kern<<<(unsigned)ntiles, TileDims<D>::TC, 0, st>>>(s.geo, P.bm, P.tbusy, P.tn, P.tf,
-                                                       (const FT*)P.tr, P.bin_cnt, (FT*)s.F);
+    auto gather = [&](auto reach) {
+      constexpr int RE = decltype(reach)::value;
+      if constexpr (D == 3) {
+        using S = StripShape<W, RE>;
+        if (strips_fit<W, RE>(s.geo)) {
+          static_assert(S::PER_TILE == S::WARPS, "one CTA per tile");
+          k_spread_strips<W, RE, FT><<<(unsigned)ntiles, S::WARPS * 32, 0, st>>>(
+              s.geo, P.bm, P.np, P.tbusy, P.tn, P.tf, (const FT*)P.tr, P.bin_cnt, (FT*)s.F,
+              s.err);
+          return;
+        }
+      }
+      k_spread_gather<D, W, RE, FT><<<(unsigned)ntiles, TileDims<D>::TC, 0, st>>>(
+          s.geo, P.bm, P.tbusy, P.tn, P.tf, (const FT*)P.tr, P.bin_cnt, (FT*)s.F);
+    };
+    if (s.phy.rebin > 1) gather(std::integral_constant<int, R0 + 1>{});
+    else gather(std::integral_constant<int, R0>{});
     if (nk) *nk += 1;
   }
   return cudaGetLastError();

@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "pibm_internal.cuh"
+#include "strips_device.cuh"
 
 namespace pibm {
 
@@ -2133,7 +2134,7 @@ __device__ __forceinline__ void spread_gather_at(const Geometry& g, const BinMap
           FT wt = r[o[0]] * r[4 + o[1]];
           if constexpr (D == 3) wt *= r[8 + o[2]];
 #pragma unroll
-          for (int k = 0; k < D; ++k) acc[k] += r[12 + k] * wt;
+          for (int k = 0; k < D; ++k) acc[k] = fma(r[12 + k], wt, acc[k]);
         }
       }
     }
@@ -2157,6 +2158,34 @@ __global__ void __launch_bounds__(TileDims<D>::TC) k_spread_gather(
   const int z = (r / bm.nt[1]) * TD::TZ + (int)threadIdx.x / (TD::TX * TD::TY);
   if (x >= g.n[0] || y >= g.n[1] || z >= g.n[2]) return;
   spread_gather_at<D, W, R, FT>(g, bm, tf, tr, start, F, x, y, z);
+}
+
+// The same sums in 3D by strips (strips_device.cuh), one warp per strip: a cell receives
+// its terms in the same order and arithmetic as from spread_gather_at, so the results
+// are equal bit for bit. Each record is read once per strip instead of once per cell (in
+// the per-cell form half of the visits miss and the lanes of a warp read different
+// records). On a 64^3 lattice with 62,500 particles in FP64 407 -> 254 us, on 96^3 with
+// 20,000 196 -> 57 us. In 2D a cell has few visitors and the strips' serial walk costs
+// more (72 x 60: 9.6 us against 5.9).
+template <int W, int R, typename FT>
+__global__ void __launch_bounds__(StripShape<W, R>::WARPS * 32) k_spread_strips(
+    Geometry g, BinMap bm, long long np, const int* __restrict__ tbusy,
+    const unsigned* __restrict__ tn, const int4* __restrict__ tf, const FT* __restrict__ tr,
+    const unsigned* __restrict__ start, FT* __restrict__ F, unsigned* __restrict__ err) {
+  using S = StripShape<W, R>;
+  __shared__ FT acc_[S::WARPS][3][S::CELLS];
+  __shared__ int2 queue[S::WARPS][S::QUEUE];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Strip st = strip_of<W, R>(g, bm, tbusy, tn[0], blockIdx.x * S::WARPS + warp);
+  if (!st.valid) return;  // the whole warp; no block-wide barrier below
+  FT(&acc)[3][S::CELLS] = acc_[warp];
+  strip_sums<W, R, FT>(g, bm, np, st, tf, tr, start, err, acc, queue[warp]);
+  for (int i = lane; i < S::CELLS; i += 32) {
+    const int x = st.x0 + i % S::SX, y = st.y0 + i / S::SX;
+    if (x >= g.n[0] || y >= g.n[1]) continue;
+    const FT v[3] = {acc[0][i], acc[1][i], acc[2][i]};
+    store_force<3, FT>(F, x + (long long)g.n[0] * (y + (long long)g.n[1] * st.z0), v);
+  }
 }
 
 // g and Fc of the last step are stored by that step's slot, which is the storage
