@@ -6,8 +6,8 @@
 // The forward run is the library's own step in deterministic mode, so a replayed
 // stretch of steps reproduces the trajectory bit for bit. Every K steps the whole
 // workspace is kept as a checkpoint; the reverse sweep replays each stretch from
-// its checkpoint, keeping a tape of the workspace as it stands before each
-// collision (stored populations of the step start, the spread force, the moment
+// its checkpoint (the last one is taped by the forward sweep itself), keeping a tape
+// of the workspace as it stands before each collision (stored populations of the step start, the spread force, the moment
 // field, the particle state of both buffers and the cell list), then runs the
 // adjoint of each step backwards:
 //   1. streaming and collision (Eqs. 2, 3, 8) per cell: the pull of the forward
@@ -20,6 +20,7 @@
 //   4. that field into the adjoint of the post-stream populations.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "pibm_internal.cuh"
@@ -90,6 +91,35 @@ __device__ __forceinline__ void axis_taps_d(double X, int n, int periodic, TapsD
   }
 }
 
+// The same from the record the forward step kept (first node and weights), for a
+// stencil that no wall clips: the four cosine weights are 1/4 (1 + c), 1/4 (1 - s),
+// 1/4 (1 - c), 1/4 (1 + s), so the first two give the sine and cosine of the derivatives
+// without evaluating them again.
+template <int W>
+__device__ __forceinline__ void axis_taps_kept(int first, const double* __restrict__ w, int n,
+                                               TapsD<W>& t) {
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    t.w[i] = w[i];
+    int k = first + i;
+    if (k < 0 || k >= n) {
+      k %= n;
+      k = k < 0 ? k + n : k;
+    }
+    t.idx[i] = k;
+  }
+  if constexpr (W == 2) {
+    t.dw[0] = -1.0;
+    t.dw[1] = 1.0;
+  } else {
+    const double c = 0.125 * 3.14159265358979323846;
+    t.dw[0] = fma(-4.0 * c, t.w[1], c);
+    t.dw[1] = fma(4.0 * c, t.w[0], -c);
+    t.dw[2] = -t.dw[0];
+    t.dw[3] = -t.dw[1];
+  }
+}
+
 // Neighbour of (x, y, z) in the direction sgn * e_a, wrapped on periodic axes;
 // false when it lies beyond a wall (the link then bounces back).
 template <int Q>
@@ -127,6 +157,7 @@ __device__ __forceinline__ void weighted_moments(const double (&v)[Q], double& m
   constexpr double w1 = L::w(1), w2 = L::w(Q - 1);
   double ax = 0.0, d0 = 0.0, dd[3] = {0.0, 0.0, 0.0}, od[3] = {0.0, 0.0, 0.0};
   double off[3] = {0.0, 0.0, 0.0}, pk[3] = {0.0, 0.0, 0.0}, mk[3] = {0.0, 0.0, 0.0};
+  bool hd[3] = {false, false, false}, ho[3] = {false, false, false};  // sums begun
 #pragma unroll
   for (int a = 1; a < Q; a += 2) {
     const double p = v[a] + v[a + 1], m = v[a] - v[a + 1];
@@ -141,16 +172,20 @@ __device__ __forceinline__ void weighted_moments(const double (&v)[Q], double& m
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       if (L::e(a, k) == 0) continue;
-      dd[k] += p;
-      od[k] += L::e(a, k) > 0 ? m : -m;
+      const double q = L::e(a, k) > 0 ? m : -m;
+      dd[k] = hd[k] ? dd[k] + p : p;
+      od[k] = hd[k] ? od[k] + q : q;
+      hd[k] = true;
     }
 #pragma unroll
     for (int k = 0; k < D; ++k)
 #pragma unroll
       for (int l = k + 1; l < D; ++l) {
-        const int s = L::e(a, k) * L::e(a, l);
-        if (s > 0) off[k + l - 1] += p;
-        if (s < 0) off[k + l - 1] -= p;
+        const int s = L::e(a, k) * L::e(a, l), i = k + l - 1;
+        if (s == 0) continue;
+        const double q = s > 0 ? p : -p;
+        off[i] = ho[i] ? off[i] + q : q;
+        ho[i] = true;
       }
   }
   m0 = L::w(0) * v[0] + (w1 * ax + w2 * d0);
@@ -177,7 +212,7 @@ __device__ __forceinline__ void weighted_moments(const double (&v)[Q], double& m
 //   jb = ub / rho, Fb = cF V + jb / 2,   rhob = om sum w gb poly - jb.u,
 //   fb = (1 - om) gb + rhob + e.jb.
 // FP64-bound: on a 96^3 D3Q19 lattice the form that summed every term per
-// velocity took 1,996 us with a separate stream pass of 371 us; now 466 us with the pull
+// velocity took 1,996 us with a separate stream pass of 371 us; now 445 us with the pull
 // included (and 48 us for the moment terms, which the stream pass used to add).
 template <int Q>
 __global__ void __launch_bounds__(ADJ_CELLS) k_adj_collide(Geometry g, double om, double cF,
@@ -226,6 +261,7 @@ __global__ void __launch_bounds__(ADJ_CELLS) k_adj_collide(Geometry g, double om
     for (int k = 0; k < D; ++k) Fv[k] = F[FS * c + k];
     // moments of the populations (stored as f - w) and sum gb s
     double dev = f[0], gs = gb[0] * f[0], j[3] = {0.0, 0.0, 0.0};
+    bool hj[3] = {false, false, false};
 #pragma unroll
     for (int a = 1; a < Q; a += 2) {
       dev += f[a] + f[a + 1];
@@ -233,10 +269,14 @@ __global__ void __launch_bounds__(ADJ_CELLS) k_adj_collide(Geometry g, double om
       gs += gb[a + 1] * f[a + 1];
       const double m = f[a] - f[a + 1];
 #pragma unroll
-      for (int k = 0; k < D; ++k)
-        if (L::e(a, k) != 0) j[k] += L::e(a, k) > 0 ? m : -m;
+      for (int k = 0; k < D; ++k) {
+        if (L::e(a, k) == 0) continue;
+        const double q = L::e(a, k) > 0 ? m : -m;
+        j[k] = hj[k] ? j[k] + q : q;
+        hj[k] = true;
+      }
     }
-    const double rho = 1.0 + dev, inv = 1.0 / rho;
+    const double rho = 1.0 + dev, inv = rcp_series(rho);
     double M0, M1[3], M2[6];
     weighted_moments<Q>(gb, M0, M1, M2);
     double u[3] = {0.0, 0.0, 0.0}, uu = 0.0, uF = 0.0;
@@ -323,6 +363,8 @@ struct AdjArgs {
   const unsigned* pid;
   const int4* cs;
   const unsigned* start;
+  const int4* tf;       // stencil records of the step's ordered spreading, by slot
+  const double* tr;
   const double* mom;    // moment field of the post-stream state [pitch][4]
   // adjoint state
   const double* Fbar;   // [pitch][FS]
@@ -346,7 +388,7 @@ struct AdjArgs {
 // particles fill the GPU, and the FP64 taps, row sums and scalar updates each run
 // on full warps. One thread per particle left most SMs with a single warp walking
 // 64 taps one after another: on 20,000 particles of a 96^3 lattice the two kernels
-// took 105 and 352 us, now 79 and 169 us.
+// took 105 and 352 us, now 74 and 153 us.
 template <int D, int W>
 struct AdjShape {
   static constexpr int WZ = D == 3 ? W : 1;
@@ -360,16 +402,22 @@ struct AdjTapsShared {
   TapsD<W> t[AdjShape<D, W>::PPB][D];
 };
 
-// Taps of the CTA's particles, one thread per particle and axis. X by storage
-// position; p[i] is particle i's (np: none).
+// Taps of the CTA's particles, one thread per particle and axis; p[i] is the storage
+// position of particle i (np: none).
 template <int D, int W>
 __device__ __forceinline__ void adj_block_taps(const AdjArgs& A, const unsigned* p,
                                                AdjTapsShared<D, W>& sh) {
   using S = AdjShape<D, W>;
   for (int i = threadIdx.x; i < S::PPB * D; i += S::THREADS) {
     const int q = i % S::PPB, k = i / S::PPB;
-    if (p[q] < (unsigned)A.np)
-      axis_taps_d<W>(A.X[k * A.np + p[q]], A.g.n[k], A.g.periodic[k], sh.t[q][k]);
+    if (p[q] >= (unsigned)A.np) continue;
+    const long long sl = blockIdx.x * (long long)S::PPB + q;
+    const int4 f = A.tf[sl];
+    const int first = k == 0 ? f.x : (k == 1 ? f.y : f.z);
+    if (A.g.periodic[k] || (first >= 0 && first <= A.g.n[k] - W))
+      axis_taps_kept<W>(first, A.tr + sl * TAP_RECORD + 4 * k, A.g.n[k], sh.t[q][k]);
+    else
+      axis_taps_d<W>(A.X[k * A.np + p[q]], A.g.n[k], 0, sh.t[q][k]);
   }
 }
 
@@ -795,6 +843,8 @@ State rebase_state(const State& s, const void* ws, void* tape) {
   P.bin_cnt = rebase(Q.bin_cnt, a, b);
   P.perm = rebase(Q.perm, a, b);
   P.block_sums = rebase(Q.block_sums, a, b);
+  P.tf = rebase(Q.tf, a, b);
+  P.tr = rebase((char*)Q.tr, a, b);
   P.tbusy = rebase(Q.tbusy, a, b);
   P.tn = rebase(Q.tn, a, b);
   return t;
@@ -821,6 +871,8 @@ cudaError_t adjoint_step(const State& T, AdjArgs A, const double* fnext, double*
   A.pid = T.p.pid[cur];
   A.cs = T.p.cs[cur];
   A.start = T.p.bin_cnt;
+  A.tf = T.p.tf;
+  A.tr = (const double*)T.p.tr;
   A.mom = (const double*)T.mom;
   k_adj_collide<Q><<<cell_blocks(g.ncell), ADJ_CELLS, 0, st>>>(
       g, T.phy.omega, T.phy.cF, (const double*)T.f[cur], (const double*)T.F, fnext, fbar, Fbar,
@@ -892,33 +944,50 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
 
   const bool grads = dtau || drho || dx0;
   Allocs al;
-  char* ckpt = grads ? al.get<char>(wsb * (size_t)nseg) : nullptr;
+  // checkpoints, and the tape of one stretch
+  char* ckpt = grads ? al.get<char>(wsb * (size_t)(nseg - 1)) : nullptr;
+  char* tape = grads ? al.get<char>(wsb * (size_t)std::min<int64_t>(K, nsteps)) : nullptr;
   double* scal = al.get<double>(sizeof(double) * 4);
-  if ((grads && !ckpt) || !scal) return PIBM_ENOMEM;
+  if ((grads && (!ckpt || !tape)) || !scal) return PIBM_ENOMEM;
 
+  // A copy of the workspace without the partner population buffer, which holds nothing
+  // between steps and is not read by a step's adjoint. The two buffers open the
+  // workspace, so the rest is one range behind the second.
+  auto copy_state = [&](char* to, const char* from) -> cudaError_t {
+    const char* ws = (const char*)v.ws;
+    const size_t f0 = (const char*)s.f[0] - ws, f1 = (const char*)s.f[1] - ws;
+    const size_t rest = (const char*)s.F - ws;
+    const size_t lo = s.cur == 0 ? f0 : f1, hi = s.cur == 0 ? f1 : wsb;
+    cudaError_t e = cudaMemcpyAsync(to + lo, from + lo, hi - lo, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess && s.cur == 0)
+      e = cudaMemcpyAsync(to + rest, from + rest, wsb - rest, cudaMemcpyDeviceToDevice, st);
+    return e;
+  };
   auto fwd_step = [&](char* tape_slot) -> cudaError_t {
     cudaError_t e;
     if ((e = launch_bin(s, st, nullptr)) != cudaSuccess) return e;
     if ((e = launch_contacts(s, st, nullptr)) != cudaSuccess) return e;
     if ((e = launch_couple(s, st, nullptr)) != cudaSuccess) return e;
-    if (tape_slot &&
-        (e = cudaMemcpyAsync(tape_slot, v.ws, wsb, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-      return e;
+    if (tape_slot && (e = copy_state(tape_slot, (const char*)v.ws)) != cudaSuccess) return e;
     if ((e = launch_collide_stream(s, st)) != cudaSuccess) return e;
     s.cur ^= 1;
     return cudaSuccess;
   };
 
-  // forward sweep with checkpoints
-  std::vector<int> par(nseg);
+  // forward sweep with checkpoints; the last stretch, which the reverse sweep starts
+  // with, keeps its tape at once
+  std::vector<int> par(nseg), step_par((size_t)std::min<int64_t>(K, nsteps));
   for (long long sg = 0; sg < nseg; ++sg) {
     par[sg] = s.cur;
-    if (grads &&
-        cudaMemcpyAsync(ckpt + wsb * sg, v.ws, wsb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+    const bool last = sg == nseg - 1;
+    if (grads && !last && copy_state(ckpt + wsb * sg, (const char*)v.ws) != cudaSuccess)
       return PIBM_ECUDA;
-    const long long n1 = sg == nseg - 1 ? nsteps : (sg + 1) * K;
-    for (long long n = sg * K; n < n1; ++n)
-      if (fwd_step(nullptr) != cudaSuccess) return PIBM_ECUDA;
+    const long long n0 = sg * K, n1 = last ? nsteps : n0 + K;
+    for (long long n = n0; n < n1; ++n) {
+      if (last) step_par[n - n0] = s.cur;
+      if (fwd_step(grads && last ? tape + wsb * (n - n0) : nullptr) != cudaSuccess)
+        return PIBM_ECUDA;
+    }
   }
   k_mean_last<<<1, ADJ_THREADS, 0, st>>>(np, d, s.p.U[s.cur], scal);
   if (cudaMemcpyAsync(loss, scal, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -927,7 +996,6 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   rc = pibm_status(hg.h);
   if (rc != PIBM_OK || !grads) return rc;
 
-  char* tape = al.get<char>(wsb * (size_t)K);
   // adjoint of the post-stream populations: of the step after (io) and of this one
   double* fb[2] = {al.get<double>(sizeof(double) * q * P), al.get<double>(sizeof(double) * q * P)};
   double* Fbar = al.get<double>(sizeof(double) * FS * P);
@@ -942,7 +1010,7 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   double* jlb = al.get<double>(sizeof(double) * d * np);
   double* mb_tmp = al.get<double>(sizeof(double) * np);
   double* drho_d = al.get<double>(sizeof(double) * np);
-  if (!tape || !fb[0] || !fb[1] || !Fbar || !rjbar || !om_part || !pb[0][0] || !pb[0][1] ||
+  if (!fb[0] || !fb[1] || !Fbar || !rjbar || !om_part || !pb[0][0] || !pb[0][1] ||
       !pb[1][0] || !pb[1][1] || !Xb_tmp || !Ub_tmp || !Fcb || !rlb || !jlb || !mb_tmp || !drho_d)
     return PIBM_ENOMEM;
   // adjoint of the final state: d loss / d U_last = 1 / np
@@ -971,16 +1039,16 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   A.rjbar = rjbar;
   A.drho = drho_d;
   A.err = s.err;
-  std::vector<int> step_par((size_t)K);
   for (long long sg = nseg - 1; sg >= 0; --sg) {
-    // replay the stretch from its checkpoint, keeping the tape
-    if (cudaMemcpyAsync(v.ws, ckpt + wsb * sg, wsb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return PIBM_ECUDA;
-    s.cur = par[sg];
-    const long long n0 = sg * K, n1 = sg == nseg - 1 ? nsteps : (sg + 1) * K;
-    for (long long n = n0; n < n1; ++n) {
-      step_par[n - n0] = s.cur;
-      if (fwd_step(tape + wsb * (n - n0)) != cudaSuccess) return PIBM_ECUDA;
+    const long long n0 = sg * K, n1 = sg == nseg - 1 ? nsteps : n0 + K;
+    if (sg < nseg - 1) {
+      // replay the stretch from its checkpoint, keeping the tape
+      s.cur = par[sg];
+      if (copy_state((char*)v.ws, ckpt + wsb * sg) != cudaSuccess) return PIBM_ECUDA;
+      for (long long n = n0; n < n1; ++n) {
+        step_par[n - n0] = s.cur;
+        if (fwd_step(tape + wsb * (n - n0)) != cudaSuccess) return PIBM_ECUDA;
+      }
     }
     for (long long n = n1 - 1; n >= n0; --n) {
       State T = rebase_state(s, v.ws, tape + wsb * (n - n0));
