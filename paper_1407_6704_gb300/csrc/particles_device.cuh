@@ -1651,9 +1651,13 @@ __global__ void __launch_bounds__(COUPLE_WARPS * 32,
 //      sums are exact (independent of their order);
 //   4. every window node with a non-zero force is added to the force field by
 //      one vector atomic, converted back to FP32.
-// Bound by shared-memory wavefronts (59 % busy at 24 warps per SM), next by the FP64
-// pipe of the update. Component-wise force planes and the update's conversions on the
-// bits took it from 1,396 to 1,197 us on the 256^3 workload.
+// Bound by shared-memory wavefronts (moment reads 27 %, force adds 21 % of the peak)
+// and the FP64 pipe of the update (26 %), with 32 warps per SM. On the 256^3 workload:
+// 1,396 us with both windows in 16-byte cells; 1,197 with component-wise force planes
+// and the update's conversions on the bits; 1,051 with the weights staged in shared
+// memory (which leaves 64 registers and a fourth CTA per SM; 1,219 with three) and the
+// spreading by columns. The gathers stay one lane per particle, in the order of
+// gather_moments: in 16-bit storage another order moves a run by its storage error.
 // The last chunk of a group takes every remaining particle; beyond 256 of them,
 // or if the box exceeds the window (a 2D group that wraps to the next tile row),
 // the CTA falls back to the direct path.
@@ -1673,13 +1677,21 @@ struct CoupleWindow {
 };
 
 template <int Q, int W, class St, typename FT, bool P64 = false>
-__global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tiles(CoupleArgs A) {
+__global__ void __launch_bounds__(256, 4) k_couple_tiles(CoupleArgs A) {
   using R = typename St::R;
   constexpr int D = Lattice<Q>::D;
   using Win = CoupleWindow<D, W>;
   static_assert(sizeof(R) == 4 && sizeof(FT) == 4, "FP32 arithmetic");
   // the moment window, reused for the force window in fixed point
   __shared__ float4 win[Win::VMAX];
+  // weights per axis, A_p g and the stencil's first node in the window, by lane
+  struct Stage {
+    float w[D][32][W], amp[32][D];
+    int base[32];
+  };
+  __shared__ Stage stages[8];
+  Stage& stage = stages[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
   __shared__ int box[6];
   __shared__ float amp_bound[8][3];  // per warp and component: sum of |A_p g_k| w_max
   const Geometry& g = A.g;
@@ -1709,7 +1721,8 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
   float4 mf = make_float4(0.f, 0.f, 0.f, 0.f);
   unsigned p = 0;
   double X[3] = {0.0, 0.0, 0.0};
-  Taps<W, R> tx, ty, tz;
+  int first[3] = {0, 0, 0};
+  float wmax = 0.f;  // largest weight product
   if (act) {
     mc = A.cs[sl];
     mf = A.xs[sl];
@@ -1719,16 +1732,34 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
       act = false;
     }
   }
-  if (act) {
-    particle_taps<D, W, false, R>(g, mc, mf, X, tx, ty, tz);
-    atomicMin(&box[0], tx.first);
-    atomicMin(&box[1], ty.first);
-    atomicMax(&box[3], tx.first + W - 1);
-    atomicMax(&box[4], ty.first + W - 1);
-    if constexpr (D == 3) {
-      atomicMin(&box[2], tz.first);
-      atomicMax(&box[5], tz.first + W - 1);
+  {
+    Taps<W, R> tx, ty, tz;
+    float mx = 0.f, my = 0.f, mz = D == 3 ? 0.f : 1.f;
+    if (act) {
+      particle_taps<D, W, false, R>(g, mc, mf, X, tx, ty, tz);
+      first[0] = tx.first;
+      first[1] = ty.first;
+      if constexpr (D == 3) first[2] = tz.first;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        atomicMin(&box[k], first[k]);
+        atomicMax(&box[3 + k], first[k] + W - 1);
+      }
     }
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const float a = act ? tx.w[i] : 0.f, b = act ? ty.w[i] : 0.f;
+      stage.w[0][lane][i] = a;
+      stage.w[1][lane][i] = b;
+      mx = fmaxf(mx, a);
+      my = fmaxf(my, b);
+      if constexpr (D == 3) {
+        const float c = act ? tz.w[i] : 0.f;
+        stage.w[D - 1][lane][i] = c;
+        mz = fmaxf(mz, c);
+      }
+    }
+    wmax = mx * my * mz;
   }
   __syncthreads();
   const int bx = box[0], by = box[1], bz = box[2];
@@ -1784,6 +1815,7 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
   }
   __syncthreads();
   // --- 2. interpolation (Eq. 4) and the particle update (Eq. 13) ---
+  const int base = ((first[2] - bz) * wy + first[1] - by) * wx + first[0] - bx;
   FT amp[3] = {FT(0), FT(0), FT(0)};
   if (act) {
     double U[3] = {0.0, 0.0, 0.0};
@@ -1799,21 +1831,16 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
     R rs = R(0), js[3] = {R(0), R(0), R(0)};
 #pragma unroll 1
     for (int iz = 0; iz < WZ; ++iz) {
-      R wzz = R(1);
-      int oz = 0;
-      if constexpr (D == 3) {
-        wzz = pick(tz.w, iz);
-        oz = (tz.first + iz - bz) * wy;
-      }
+      const R wzz = D == 3 ? stage.w[D - 1][lane][iz] : R(1);
       if (wzz == R(0)) continue;
 #pragma unroll
       for (int iy = 0; iy < W; ++iy) {
-        const R wyz = ty.w[iy] * wzz;
-        const int row = (oz + ty.first + iy - by) * wx + tx.first - bx;
+        const R wyz = stage.w[1][lane][iy] * wzz;
+        const float4* row = win + base + (iz * wy + iy) * wx;
 #pragma unroll
         for (int ix = 0; ix < W; ++ix) {
-          const float4 m = win[row + ix];
-          const R wt = tx.w[ix] * wyz;
+          const float4 m = row[ix];
+          const R wt = stage.w[0][lane][ix] * wyz;
           rs += wt * m.x;
           js[0] += wt * m.y;
           js[1] += wt * m.z;
@@ -1823,26 +1850,13 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
     }
     advance_particle<D, St, FT, P64, FCT>(A, sl, p, mc, mf, X, U, Fc, rs, js, amp);
   }
+  stage.base[lane] = base;
   // the fixed-point scales: per component, a bound on every node's |sum|
   {
-    float wm = 0.f;
-    if (act) {
-      float mx = 0.f, my = 0.f, mz = 1.f;
-#pragma unroll
-      for (int i = 0; i < W; ++i) {
-        mx = fmaxf(mx, tx.w[i]);
-        my = fmaxf(my, ty.w[i]);
-      }
-      if constexpr (D == 3) {
-        mz = 0.f;
-#pragma unroll
-        for (int i = 0; i < W; ++i) mz = fmaxf(mz, tz.w[i]);
-      }
-      wm = mx * my * mz;
-    }
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      float b = fabsf(amp[k]) * wm;
+      stage.amp[lane][k] = amp[k];
+      float b = fabsf(amp[k]) * wmax;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
       if ((threadIdx.x & 31) == 0) amp_bound[threadIdx.x >> 5][k] = b;
@@ -1871,28 +1885,29 @@ __global__ void __launch_bounds__(256, Lattice<Q>::D == 3 ? 3 : 4) k_couple_tile
   int* wi = reinterpret_cast<int*>(win);
   for (int v = threadIdx.x; v < D * V; v += blockDim.x) wi[v] = 0;
   __syncthreads();
-  if (act) {
+  // W neighbouring lanes take a particle's stencil by columns, 32 / W particles per
+  // round: the adds of a row go to W consecutive words. A scale is a power of two, so it
+  // is multiplied in before the weight without changing the rounding.
+#pragma unroll 1
+  for (int r = 0; r < W; ++r) {
+    const int src = r * (32 / W) + lane / W, ix = lane % W;
+    const float wxs = stage.w[0][src][ix];
+    if (wxs == 0.f) continue;  // a dropped node, or no particle
+    float a[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) a[k] = stage.amp[src][k] * scale[k];
+    int* cell = wi + stage.base[src] + ix;
 #pragma unroll 1
     for (int iz = 0; iz < WZ; ++iz) {
-      FT wzz = FT(1);
-      int oz = 0;
-      if constexpr (D == 3) {
-        wzz = (FT)pick(tz.w, iz);
-        oz = (tz.first + iz - bz) * wy;
-      }
-      if (wzz == FT(0)) continue;
+      const float wzz = D == 3 ? stage.w[D - 1][src][iz] : 1.f;
 #pragma unroll
       for (int iy = 0; iy < W; ++iy) {
-        const FT wyz = (FT)ty.w[iy] * wzz;
-        const int row = (oz + ty.first + iy - by) * wx + tx.first - bx;
+        const float wyz = stage.w[1][src][iy] * wzz;
+        const float wt = wxs * wyz;
+        if (wt == 0.f) continue;
+        int* c = cell + (iz * wy + iy) * wx;
 #pragma unroll
-        for (int ix = 0; ix < W; ++ix) {
-          const FT wt = (FT)tx.w[ix] * wyz;
-          if (wt == FT(0)) continue;
-#pragma unroll
-          for (int k = 0; k < D; ++k)
-            atomicAdd(wi + k * V + row + ix, __float2int_rn(amp[k] * wt * scale[k]));
-        }
+        for (int k = 0; k < D; ++k) atomicAdd(c + k * V, __float2int_rn(a[k] * wt));
       }
     }
   }
