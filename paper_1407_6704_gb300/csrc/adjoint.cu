@@ -892,21 +892,43 @@ cudaError_t adjoint_step_w(const State& T, const AdjArgs& A, const double* fnext
                           : adjoint_step<Q, 4>(T, A, fnext, fbar, Fbar, om_part, st);
 }
 
-// Device allocations of the gradient run, released together.
-struct Allocs {
-  std::vector<void*> ptrs;
-  ~Allocs() {
-    for (void* p : ptrs) cudaFree(p);
+// One device allocation for everything a gradient run needs, laid out by walking the
+// same list of arrays twice: once to add up the bytes, once for the pointers.
+struct Arena {
+  char* base = nullptr;
+  size_t bytes = 0;
+  bool counting = true;
+  ~Arena() {
+    if (base) cudaFree(base);
   }
   template <typename T>
-  T* get(size_t bytes) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, bytes ? bytes : 256) != cudaSuccess) {
+  T* take(size_t n) {
+    T* p = counting ? nullptr : (T*)(base + bytes);
+    bytes += (n + 255) / 256 * 256;
+    return p;
+  }
+  bool allocate() {
+    if (cudaMalloc(&base, bytes ? bytes : 256) != cudaSuccess) {
       cudaGetLastError();
-      return nullptr;
+      base = nullptr;
+      return false;
     }
-    ptrs.push_back(p);
-    return (T*)p;
+    counting = false;
+    bytes = 0;
+    return true;
+  }
+};
+
+// CUDA graphs of the recurring stretches (forward, replay, reverse), by the parity they
+// start from.
+struct StretchGraphs {
+  cudaStream_t cap = nullptr;
+  cudaGraphExec_t exec[3][2] = {};
+  ~StretchGraphs() {
+    for (auto& k : exec)
+      for (cudaGraphExec_t e : k)
+        if (e) cudaGraphExecDestroy(e);
+    if (cap) cudaStreamDestroy(cap);
   }
 };
 
@@ -930,30 +952,56 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   pibm_config cfg = *cfg_in;
   cfg.deterministic = 1;  // replayed stretches reproduce the forward run bit for bit
   cudaStream_t st = (cudaStream_t)stream;
-  HandleGuard hg;
-  int rc = pibm_create(&cfg, nullptr, 0, stream, &hg.h);
+  size_t wsb = 0;
+  int rc = pibm_workspace_bytes(&cfg, &wsb);
+  if (rc != PIBM_OK) return rc;
+  const bool grads = dtau || drho || dx0;
+  const int d = cfg.lattice == PIBM_D2Q9 ? 2 : 3, q = cfg.lattice, FS = d == 2 ? 2 : 4;
+  const long long np = cfg.n_particles, ncell = cfg.n[0] * cfg.n[1] * cfg.n[2];
+  const long long P = (ncell + 63) / 64 * 64;  // the plane pitch
+  const long long nseg = (nsteps + K - 1) / K;
+  const size_t D8 = sizeof(double);
+
+  Arena al;
+  char *ws, *ckpt = nullptr, *tape = nullptr;
+  double *scal, *fb[2], *Fbar, *rjbar, *om_part, *pb[2][2], *Xb_tmp, *Ub_tmp, *Fcb, *rlb, *jlb,
+      *mb_tmp, *drho_d;
+  for (int pass = 0; pass < 2; ++pass) {
+    ws = al.take<char>(wsb);
+    scal = al.take<double>(D8 * 4);
+    if (grads) {
+      // checkpoints, the tape of one stretch, and the adjoint state: of the post-stream
+      // populations (of the step after and of this one), the force, the moment field
+      // and the particles
+      ckpt = al.take<char>(wsb * (size_t)(nseg - 1));
+      tape = al.take<char>(wsb * (size_t)std::min<int64_t>(K, nsteps));
+      for (int i = 0; i < 2; ++i) {
+        fb[i] = al.take<double>(D8 * q * P);
+        for (int j = 0; j < 2; ++j) pb[i][j] = al.take<double>(D8 * d * np);
+      }
+      Fbar = al.take<double>(D8 * FS * P);
+      rjbar = al.take<double>(D8 * 4 * P);
+      om_part = al.take<double>(D8 * cell_blocks(ncell));
+      Xb_tmp = al.take<double>(D8 * d * np);
+      Ub_tmp = al.take<double>(D8 * d * np);
+      Fcb = al.take<double>(D8 * d * np);
+      rlb = al.take<double>(D8 * np);
+      jlb = al.take<double>(D8 * d * np);
+      mb_tmp = al.take<double>(D8 * np);
+      drho_d = al.take<double>(D8 * np);
+    }
+    if (pass == 0 && !al.allocate()) return PIBM_ENOMEM;
+  }
+  HandleGuard hg;  // destroyed before the arena
+  rc = pibm_create(&cfg, ws, wsb, stream, &hg.h);
   if (rc != PIBM_OK) return rc;
   HandleView v = handle_view(hg.h);
   State& s = *v.s;
-  const long long np = s.p.np;
-  const int d = s.geo.d, q = s.geo.q;
-  const long long nseg = (nsteps + K - 1) / K;
-  const size_t wsb = v.ws_bytes;
-  const long long P = s.geo.pitch;
-  const int FS = d == 2 ? 2 : 4;
-
-  const bool grads = dtau || drho || dx0;
-  Allocs al;
-  // checkpoints, and the tape of one stretch
-  char* ckpt = grads ? al.get<char>(wsb * (size_t)(nseg - 1)) : nullptr;
-  char* tape = grads ? al.get<char>(wsb * (size_t)std::min<int64_t>(K, nsteps)) : nullptr;
-  double* scal = al.get<double>(sizeof(double) * 4);
-  if ((grads && (!ckpt || !tape)) || !scal) return PIBM_ENOMEM;
 
   // A copy of the workspace without the partner population buffer, which holds nothing
   // between steps and is not read by a step's adjoint. The two buffers open the
   // workspace, so the rest is one range behind the second.
-  auto copy_state = [&](char* to, const char* from) -> cudaError_t {
+  auto copy_state = [&](char* to, const char* from, cudaStream_t st) -> cudaError_t {
     const char* ws = (const char*)v.ws;
     const size_t f0 = (const char*)s.f[0] - ws, f1 = (const char*)s.f[1] - ws;
     const size_t rest = (const char*)s.F - ws;
@@ -963,31 +1011,97 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
       e = cudaMemcpyAsync(to + rest, from + rest, wsb - rest, cudaMemcpyDeviceToDevice, st);
     return e;
   };
-  auto fwd_step = [&](char* tape_slot) -> cudaError_t {
+  auto fwd_step = [&](char* tape_slot, cudaStream_t st) -> cudaError_t {
     cudaError_t e;
     if ((e = launch_bin(s, st, nullptr)) != cudaSuccess) return e;
     if ((e = launch_contacts(s, st, nullptr)) != cudaSuccess) return e;
     if ((e = launch_couple(s, st, nullptr)) != cudaSuccess) return e;
-    if (tape_slot && (e = copy_state(tape_slot, (const char*)v.ws)) != cudaSuccess) return e;
+    if (tape_slot && (e = copy_state(tape_slot, (const char*)v.ws, st)) != cudaSuccess) return e;
     if ((e = launch_collide_stream(s, st)) != cudaSuccess) return e;
     s.cur ^= 1;
     return cudaSuccess;
   };
+  int io = 0;  // pb[io], fb[io] = adjoint of the state being reversed into
+  // n forward steps, taped or not
+  auto forward = [&](long long n, bool taped, cudaStream_t st) -> cudaError_t {
+    for (long long i = 0; i < n; ++i) {
+      const cudaError_t e = fwd_step(taped ? tape + wsb * i : nullptr, st);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  };
+  AdjArgs A{};
+  // the adjoint of the n steps on the tape, whose first started from buffer par
+  auto reverse = [&](long long n, int par, cudaStream_t st) -> cudaError_t {
+    for (long long i = n - 1; i >= 0; --i) {
+      State T = rebase_state(s, v.ws, tape + wsb * i);
+      T.cur = par ^ (int)(i & 1);
+      A.Xb_in = pb[io][0];
+      A.Ub_in = pb[io][1];
+      A.Xb_out = pb[1 - io][0];
+      A.Ub_out = pb[1 - io][1];
+      cudaError_t e = cudaErrorInvalidValue;
+      if (q == 9) e = adjoint_step_w<9>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
+      else if (q == 15) e = adjoint_step_w<15>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
+      else if (q == 19) e = adjoint_step_w<19>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
+      if (e != cudaSuccess) return e;
+      io = 1 - io;
+    }
+    return cudaSuccess;
+  };
+  // Full stretches recur with the same arguments (up to the buffer parity they start
+  // from), so from the fourth stretch on they are captured once and replayed: a step of a
+  // small lattice is 13 launches of a few microseconds each, and launching them one by
+  // one took longer than running them (72 x 60, 120 steps: 23.3 ms for 14.9 ms of
+  // kernels).
+  StretchGraphs graphs;
+  bool replayed = grads && nseg >= 4 && K <= 64 &&
+                  cudaStreamCreateWithFlags(&graphs.cap, cudaStreamNonBlocking) == cudaSuccess;
+  // body(stream) enqueues stretch kind kd of K steps starting from parity key; the host
+  // state it advances is s.cur (forward kinds) or io (reverse)
+  auto stretch = [&](int kd, int key, auto&& body) -> cudaError_t {
+    if (!replayed) return body(st);
+    int& moved = kd == 2 ? io : s.cur;
+    const int before = moved;
+    cudaGraphExec_t& ex = graphs.exec[kd][key];
+    if (!ex) {
+      cudaGraph_t gr = nullptr;
+      cudaError_t e = cudaStreamBeginCapture(graphs.cap, cudaStreamCaptureModeThreadLocal);
+      if (e == cudaSuccess) {
+        e = body(graphs.cap);
+        const cudaError_t ee = cudaStreamEndCapture(graphs.cap, &gr);
+        if (e == cudaSuccess) e = ee;
+      }
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, gr, 0);
+      if (gr) cudaGraphDestroy(gr);
+      moved = before;
+      if (e != cudaSuccess) {  // not capturable here: launch directly from now on
+        cudaGetLastError();
+        ex = nullptr;
+        replayed = false;
+        return body(st);
+      }
+    }
+    moved = before ^ (int)(K & 1);
+    return cudaGraphLaunch(ex, st);
+  };
 
   // forward sweep with checkpoints; the last stretch, which the reverse sweep starts
   // with, keeps its tape at once
-  std::vector<int> par(nseg), step_par((size_t)std::min<int64_t>(K, nsteps));
+  std::vector<int> par(nseg);
   for (long long sg = 0; sg < nseg; ++sg) {
     par[sg] = s.cur;
     const bool last = sg == nseg - 1;
-    if (grads && !last && copy_state(ckpt + wsb * sg, (const char*)v.ws) != cudaSuccess)
-      return PIBM_ECUDA;
-    const long long n0 = sg * K, n1 = last ? nsteps : n0 + K;
-    for (long long n = n0; n < n1; ++n) {
-      if (last) step_par[n - n0] = s.cur;
-      if (fwd_step(grads && last ? tape + wsb * (n - n0) : nullptr) != cudaSuccess)
-        return PIBM_ECUDA;
+    const long long n = last ? nsteps - sg * K : K;
+    cudaError_t e;
+    if (last) {
+      e = forward(n, grads, st);
+    } else {
+      e = grads ? copy_state(ckpt + wsb * sg, (const char*)v.ws, st) : cudaSuccess;
+      if (e == cudaSuccess)
+        e = stretch(0, s.cur, [&](cudaStream_t to) { return forward(n, false, to); });
     }
+    if (e != cudaSuccess) return PIBM_ECUDA;
   }
   k_mean_last<<<1, ADJ_THREADS, 0, st>>>(np, d, s.p.U[s.cur], scal);
   if (cudaMemcpyAsync(loss, scal, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -996,35 +1110,16 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   rc = pibm_status(hg.h);
   if (rc != PIBM_OK || !grads) return rc;
 
-  // adjoint of the post-stream populations: of the step after (io) and of this one
-  double* fb[2] = {al.get<double>(sizeof(double) * q * P), al.get<double>(sizeof(double) * q * P)};
-  double* Fbar = al.get<double>(sizeof(double) * FS * P);
-  double* rjbar = al.get<double>(sizeof(double) * 4 * P);
-  double* om_part = al.get<double>(sizeof(double) * cell_blocks(s.geo.ncell));
-  double* pb[2][2] = {{al.get<double>(sizeof(double) * d * np), al.get<double>(sizeof(double) * d * np)},
-                      {al.get<double>(sizeof(double) * d * np), al.get<double>(sizeof(double) * d * np)}};
-  double* Xb_tmp = al.get<double>(sizeof(double) * d * np);
-  double* Ub_tmp = al.get<double>(sizeof(double) * d * np);
-  double* Fcb = al.get<double>(sizeof(double) * d * np);
-  double* rlb = al.get<double>(sizeof(double) * np);
-  double* jlb = al.get<double>(sizeof(double) * d * np);
-  double* mb_tmp = al.get<double>(sizeof(double) * np);
-  double* drho_d = al.get<double>(sizeof(double) * np);
-  if (!fb[0] || !fb[1] || !Fbar || !rjbar || !om_part || !pb[0][0] || !pb[0][1] ||
-      !pb[1][0] || !pb[1][1] || !Xb_tmp || !Ub_tmp || !Fcb || !rlb || !jlb || !mb_tmp || !drho_d)
-    return PIBM_ENOMEM;
   // adjoint of the final state: d loss / d U_last = 1 / np
-  int io = 0;  // pb[io], fb[io] = adjoint of the state being reversed into
   if (cudaMemsetAsync(fb[io], 0, sizeof(double) * q * P, st) != cudaSuccess ||
       cudaMemsetAsync(rjbar, 0, sizeof(double) * 4 * P, st) != cudaSuccess ||
       cudaMemsetAsync(pb[io][0], 0, sizeof(double) * d * np, st) != cudaSuccess ||
       cudaMemsetAsync(pb[io][1], 0, sizeof(double) * d * np, st) != cudaSuccess ||
-      cudaMemsetAsync(om_part, 0, sizeof(double) * cell_blocks(s.geo.ncell), st) != cudaSuccess ||
+      cudaMemsetAsync(om_part, 0, sizeof(double) * cell_blocks(ncell), st) != cudaSuccess ||
       cudaMemsetAsync(drho_d, 0, sizeof(double) * np, st) != cudaSuccess)
     return PIBM_ECUDA;
   k_adj_seed<<<nblk(np), ADJ_THREADS, 0, st>>>(np, d, pb[io][1]);
 
-  AdjArgs A{};
   A.g = s.geo;
   A.ph = s.phy;
   A.bm = s.p.bm;
@@ -1040,32 +1135,25 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   A.drho = drho_d;
   A.err = s.err;
   for (long long sg = nseg - 1; sg >= 0; --sg) {
-    const long long n0 = sg * K, n1 = sg == nseg - 1 ? nsteps : n0 + K;
-    if (sg < nseg - 1) {
+    const bool last = sg == nseg - 1;
+    const long long n = last ? nsteps - sg * K : K;
+    cudaError_t e = cudaSuccess;
+    if (!last) {
       // replay the stretch from its checkpoint, keeping the tape
       s.cur = par[sg];
-      if (copy_state((char*)v.ws, ckpt + wsb * sg) != cudaSuccess) return PIBM_ECUDA;
-      for (long long n = n0; n < n1; ++n) {
-        step_par[n - n0] = s.cur;
-        if (fwd_step(tape + wsb * (n - n0)) != cudaSuccess) return PIBM_ECUDA;
-      }
+      e = copy_state((char*)v.ws, ckpt + wsb * sg, st);
+      if (e == cudaSuccess)
+        e = stretch(1, par[sg], [&](cudaStream_t to) { return forward(n, true, to); });
     }
-    for (long long n = n1 - 1; n >= n0; --n) {
-      State T = rebase_state(s, v.ws, tape + wsb * (n - n0));
-      T.cur = step_par[n - n0];
-      A.Xb_in = pb[io][0];
-      A.Ub_in = pb[io][1];
-      A.Xb_out = pb[1 - io][0];
-      A.Ub_out = pb[1 - io][1];
-      cudaError_t e = cudaErrorInvalidValue;
-      if (q == 9) e = adjoint_step_w<9>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
-      else if (q == 15) e = adjoint_step_w<15>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
-      else if (q == 19) e = adjoint_step_w<19>(T, A, fb[io], fb[1 - io], Fbar, om_part, st);
-      if (e != cudaSuccess) return PIBM_ECUDA;
-      io = 1 - io;
+    // the adjoint buffers alternate with the tape's parity (both flip with every step
+    // from the last one back), so that parity is the whole key of a reverse stretch
+    if (e == cudaSuccess) {
+      if (n == K) e = stretch(2, par[sg], [&](cudaStream_t to) { return reverse(n, par[sg], to); });
+      else e = reverse(n, par[sg], st);
     }
+    if (e != cudaSuccess) return PIBM_ECUDA;
   }
-  k_sum_blocks<<<1, ADJ_THREADS, 0, st>>>(cell_blocks(s.geo.ncell), om_part, scal + 1);
+  k_sum_blocks<<<1, ADJ_THREADS, 0, st>>>(cell_blocks(ncell), om_part, scal + 1);
   double omb = 0.0;
   if (cudaMemcpyAsync(&omb, scal + 1, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return PIBM_ECUDA;
