@@ -1171,6 +1171,53 @@ __device__ __forceinline__ void stage_taps(TapStage<D, WI, R>& st, int lane, boo
   }
 }
 
+// The taps of PPW < 32 particles with a lane per particle and axis: on a few particles
+// the coupling is a chain of dependent operations, and the axes' sines and cosines one
+// after another are a quarter of it. An axis whose nodes fall outside the lattice (an
+// internal error) gets zero weights.
+template <int D, int WI, bool LAG, typename R, int PPW>
+__device__ __forceinline__ void stage_taps_by_axis(const CoupleArgs& A, TapStage<D, WI, R>& st,
+                                                   long long sl0, int lane) {
+  const Geometry& g = A.g;
+#pragma unroll
+  for (int u = 0; u < (D * PPW + 31) / 32; ++u) {
+    const int i = u * 32 + lane;
+    const int q = i % PPW, k = i / PPW;
+    if (k >= D) continue;
+    const long long sl = sl0 + q;
+    Taps<WI, R> t;
+    bool on = false;
+    if (sl < A.np) {
+      const int4 mc = A.cs[sl];
+      const float4 mf = A.xs[sl];
+      const unsigned p = (unsigned)mc.w;
+      const int n = k == 0 ? g.n[0] : (k == 1 ? g.n[1] : g.n[2]);
+      const int per = k == 0 ? g.periodic[0] : (k == 1 ? g.periodic[1] : g.periodic[2]);
+      if (p < (unsigned)A.np) {
+        if constexpr (sizeof(R) == 4) {
+          const int c = k == 0 ? mc.x : (k == 1 ? mc.y : mc.z);
+          const float f = k == 0 ? mf.x : (k == 1 ? mf.y : mf.z);
+          if constexpr (LAG) axis_lagrange_local(c, f, n, per, t);
+          else axis_taps_local<WI>(c, f, n, per, t);
+        } else {
+          const double x = A.X[k * A.np + p];
+          if constexpr (LAG) axis_lagrange<R>(x, n, per, t);
+          else axis_taps<WI, R>(x, n, per, t);
+        }
+        on = true;
+#pragma unroll
+        for (int j = 0; j < WI; ++j) on = on && (unsigned)t.idx[j] < (unsigned)n;
+        if (!on) atomicOr(A.err, ERR_INDEX);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < WI; ++j) {
+      st.w[k][q][j] = on ? t.w[j] : R(0);
+      st.idx[k][q][j] = on ? t.idx[j] : 0;
+    }
+  }
+}
+
 // Eq. (4) on the moments of the warp's particles: rs = sum w (rho - S) and js =
 // sum w j of this lane's particle, from the staged taps. Each lane sums its column
 // over the rows, weights it, and the columns are added in a fixed order. ROUNDS:
@@ -1490,7 +1537,10 @@ __device__ __forceinline__ void couple_warp(const CoupleArgs& A, long long sl0,
     }
   }
   // --- interpolation of rho, j (Eq. 4) ---
-  {
+  __syncwarp();  // the stage may still be read for the warp's previous particles
+  if constexpr (PPW < 32) {
+    stage_taps_by_axis<D, WI, LAG, R, PPW>(A, stage.in, sl0, lane);
+  } else {
     Taps<WI, R> tx, ty, tz;
     bool on = act;
     if (act) {
@@ -1500,7 +1550,6 @@ __device__ __forceinline__ void couple_warp(const CoupleArgs& A, long long sl0,
         on = false;
       }
     }
-    __syncwarp();  // the stage may still be read for the warp's previous particles
     stage_taps<D, WI, R>(stage.in, lane, on, tx, ty, tz);
   }
   __syncwarp();
@@ -1612,7 +1661,7 @@ __device__ __forceinline__ void couple_slots(const CoupleArgs& A, long long sl0,
     couple_at<Q, W, St, FT, LAG, NC, P64>(A, sl0 + (threadIdx.x & 31));
 }
 
-// Warps per CTA; PPW particles each.
+// Warps per CTA at most (warps_per_cta); PPW particles each.
 constexpr int COUPLE_WARPS = 8;
 
 template <int Q, int W, class St, typename FT, bool LAG, bool P64, int PPW>
@@ -1620,9 +1669,9 @@ __global__ void __launch_bounds__(COUPLE_WARPS * 32,
                                   sizeof(typename St::R) == 4 ? (Lattice<Q>::D == 2 ? 5 : 4) : 2)
     k_couple(CoupleArgs A) {
   __shared__ CoupleStage<Q, W, St, LAG> stage[COUPLE_WARPS];
-  const int w = threadIdx.x >> 5;
-  couple_slots<Q, W, St, FT, LAG, true, P64, PPW>(
-      A, (blockIdx.x * (long long)COUPLE_WARPS + w) * PPW, stage[w]);
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  couple_slots<Q, W, St, FT, LAG, true, P64, PPW>(A, (blockIdx.x * (long long)nw + w) * PPW,
+                                                  stage[w]);
 }
 
 // Coupling by tiles (32- and 16-bit storage, delta interpolation, atomic
