@@ -37,6 +37,13 @@ def test_fields_match_numpy(lattice, n, periodic, precision):
     r = sim.read("rho", "j", "pop")
     wb = w.reshape((-1,) + (1,) * d)
     assert np.all(np.abs(r["pop"] - f0) <= REL[precision] * np.abs(f0 - wb) + 2.0 ** -36 + 4e-16)
+    # the read-back adds w to the stored value, widened exactly
+    dev = f0 - wb
+    stored = {"fp64": lambda: dev, "fp32": lambda: dev.astype(np.float32).astype(np.float64),
+              "fp16": lambda: (dev.astype(np.float32) * np.float32(4096)).astype(np.float16)
+              .astype(np.float64) / 4096,
+              "bf16": lambda: torch.from_numpy(dev.astype(np.float32)).bfloat16().double().numpy()}
+    assert np.array_equal(r["pop"], stored[precision]() + wb)
     # rho and j are sums of at most q FP64 terms of size at most max(f)
     tol = 2 * q * 2.0 ** -52
     assert np.abs(r["rho"] - r["pop"].sum(0)).max() <= tol
