@@ -1017,7 +1017,7 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
     if ((e = launch_contacts(s, st, nullptr)) != cudaSuccess) return e;
     if ((e = launch_couple(s, st, nullptr)) != cudaSuccess) return e;
     if (tape_slot && (e = copy_state(tape_slot, (const char*)v.ws, st)) != cudaSuccess) return e;
-    if ((e = launch_collide_stream(s, st)) != cudaSuccess) return e;
+    if ((e = launch_collide_stream(s, st, true)) != cudaSuccess) return e;
     s.cur ^= 1;
     return cudaSuccess;
   };

@@ -267,7 +267,7 @@ int enqueue_step(pibm_t* h, cudaStream_t st, int* nk_out, bool split_ok = true) 
   } else {
     PHASE(launch_contacts(s, st, &nk));
     PHASE(launch_couple(s, st, &nk));
-    PHASE(launch_collide_stream(s, st));
+    PHASE(launch_collide_stream(s, st, true));
     nk += 1;
   }
   s.cur ^= 1;
@@ -838,7 +838,7 @@ int pibm_autotune(pibm_t* h, int* block_xy) {
   for (int i = 0; i < ncand && rc == PIBM_OK; ++i) {
     s.cblk[0] = pk ? pair[i][0] : scal[i][0];
     s.cblk[1] = pk ? pair[i][1] : scal[i][1];
-    cudaError_t le = launch_collide_stream(s, st);
+    cudaError_t le = launch_collide_stream(s, st, false);
     if (le != cudaSuccess) {  // a shape this launch cannot take: skip it
       cudaGetLastError();
       continue;
@@ -849,7 +849,7 @@ int pibm_autotune(pibm_t* h, int* block_xy) {
       break;
     }
     for (int r = 0; r < 3; ++r)
-      if ((le = launch_collide_stream(s, st)) != cudaSuccess) {
+      if ((le = launch_collide_stream(s, st, false)) != cudaSuccess) {
         record_error("launch_collide_stream", le);
         rc = PIBM_ECUDA;
       }
@@ -1290,7 +1290,7 @@ int pibm_profile_steps(pibm_t* h, int64_t nsteps, double* phase_ms) {
           launch_contacts(s, st, &nk) != cudaSuccess ||
           cudaEventRecord(e[1], st) != cudaSuccess ||
           launch_couple(s, st, &nk) != cudaSuccess || cudaEventRecord(e[2], st) != cudaSuccess ||
-          launch_collide_stream(s, st) != cudaSuccess ||
+          launch_collide_stream(s, st, true) != cudaSuccess ||
           cudaEventRecord(e[3], st) != cudaSuccess) {
         rc = PIBM_ECUDA;
         break;

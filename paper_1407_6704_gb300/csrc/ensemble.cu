@@ -472,8 +472,9 @@ __global__ void __launch_bounds__(ENS_THREADS, EnsShape<Q, St>::MINB) k_ensemble
         R sv[Q], Fv[3] = {R(0), R(0), R(0)};
         pull_cell<Q, St>((const T*)sA.f, sA.g, x, y, z, sv);
         if (busy) take_force<D, FT, R>((FT*)sA.F, (long long)cu, Fv);
-        collide_store<Q, St>((T*)sX.fout[cur], sA.g, (long long)cu, sv, Fv, (R)sA.ph.omega,
-                             (R)sA.ph.cF, sA.err);
+        collide_store_near<Q, St, 0, false>((T*)sX.fout[cur], sA.g, (long long)cu, sv, Fv,
+                                            (R)sA.ph.omega, (R)sA.ph.cF, sA.err,
+                                            (const R*)sA.mom, busy);
         x += ENS_THREADS;
         while (x >= (int)n0) {
           x -= (int)n0;

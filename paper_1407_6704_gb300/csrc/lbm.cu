@@ -16,6 +16,8 @@ namespace pibm {
 namespace {
 
 // Pull-stream, collide, store; one thread per cell. FT: type of the force field.
+// mom, tflag, bm: the moment field and the busy flags of the tiles when both belong to
+// this step (FP64 storage; else null).
 template <int Q, class St, typename FT>
 __global__ void __launch_bounds__(256, (Lattice<Q>::D == 3 && sizeof(typename St::T) == 4) ? 5 : 0)
     k_collide_stream(const typename St::T* __restrict__ fin,
@@ -23,12 +25,19 @@ __global__ void __launch_bounds__(256, (Lattice<Q>::D == 3 && sizeof(typename St
                                                         FT* __restrict__ F, Geometry g,
                                                         typename St::R om,
                                                         typename St::R cF,
-                                                        unsigned* __restrict__ err) {
+                                                        unsigned* __restrict__ err,
+                                                        const typename St::R* mom,
+                                                        const int* __restrict__ tflag,
+                                                        BinMap bm) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= g.n[0] || y >= g.n[1]) return;
-  collide_stream_at<Q, St, FT>(fin, fout, F, g, om, cF, err, x, y, z);
+  using TD = TileDims<Lattice<Q>::D>;
+  bool busy = false;
+  if constexpr (sizeof(typename St::T) == 8)
+    busy = mom && tflag[x / TD::TX + bm.nt[0] * (y / TD::TY + bm.nt[1] * (z / TD::TZ))];
+  collide_stream_at<Q, St, FT>(fin, fout, F, g, om, cF, err, x, y, z, mom, busy);
 }
 
 // The same over the tiles of one list (the busy or the free tiles of the cell
@@ -41,7 +50,7 @@ __global__ void __launch_bounds__(TileDims<Lattice<Q>::D>::TC,
     k_collide_tiles(const typename St::T* __restrict__ fin, typename St::T* __restrict__ fout,
                     FT* __restrict__ F, Geometry g, BinMap bm, const int* __restrict__ tiles,
                     const unsigned* __restrict__ tn, int which, typename St::R om,
-                    typename St::R cF, unsigned* __restrict__ err) {
+                    typename St::R cF, unsigned* __restrict__ err, const typename St::R* mom) {
   using TD = TileDims<Lattice<Q>::D>;
   const int n = (int)tn[which];
   const int lx = threadIdx.x % TD::TX, ly = (threadIdx.x / TD::TX) % TD::TY,
@@ -55,7 +64,8 @@ __global__ void __launch_bounds__(TileDims<Lattice<Q>::D>::TC,
     const int y = (r % bm.nt[1]) * TD::TY + ly;
     const int z = (r / bm.nt[1]) * TD::TZ + lz;
     if (x < g.n[0] && y < g.n[1] && z < g.n[2])
-      collide_stream_at<Q, St, FT, HINT, NOF>(fin, fout, F, g, om, cF, err, x, y, z);
+      collide_stream_at<Q, St, FT, HINT, NOF>(fin, fout, F, g, om, cF, err, x, y, z, mom,
+                                              mom != nullptr);
     t = next;
   }
 }
@@ -355,7 +365,7 @@ dim3 collide_block(const State& s, bool pair) {
 }
 
 template <int Q, class St, typename FT>
-cudaError_t collide_stream_t(const State& s, cudaStream_t st) {
+cudaError_t collide_stream_t(const State& s, cudaStream_t st, bool moments) {
   const Geometry& g = s.geo;
   using T = typename St::T;
   using R = typename St::R;
@@ -376,9 +386,10 @@ cudaError_t collide_stream_t(const State& s, cudaStream_t st) {
   }
   dim3 blk = collide_block(s, false);
   dim3 grd((g.n[0] + blk.x - 1) / blk.x, (g.n[1] + blk.y - 1) / blk.y, g.n[2]);
+  const R* mom = sizeof(T) == 8 && moments && s.p.np > 0 ? (const R*)s.mom : nullptr;
   k_collide_stream<Q, St, FT><<<grd, blk, 0, st>>>((const T*)s.f[s.cur], (T*)s.f[1 - s.cur],
                                                    (FT*)s.F, g, (R)s.phy.omega, (R)s.phy.cF,
-                                                   s.err);
+                                                   s.err, mom, s.p.tflag, s.p.bm);
   return cudaGetLastError();
 }
 
@@ -454,7 +465,8 @@ cudaError_t launch_collide_tiles(const State& s, cudaStream_t st, int which, int
     if ((e = full_grid(kern, TC, grid)) != cudaSuccess) return e;
     kern<<<grid, TC, 0, st>>>((const T*)s.f[s.cur], (T*)s.f[1 - s.cur], (FT*)s.F, s.geo, P.bm,
                               which == 0 ? P.tbusy : P.tfree, P.tn, which, (R)s.phy.omega,
-                              (R)s.phy.cF, s.err);
+                              (R)s.phy.cF, s.err,
+                              sizeof(T) == 8 && which == 0 ? (const R*)s.mom : nullptr);
     return cudaGetLastError();
   });
 }
@@ -463,10 +475,10 @@ bool collide_uses_pair_kernel(const State& s) {
   return (s.precision == PIBM_FP16 || s.precision == PIBM_BF16) && (s.geo.n[0] & 1) == 0;
 }
 
-cudaError_t launch_collide_stream(const State& s, cudaStream_t st) {
+cudaError_t launch_collide_stream(const State& s, cudaStream_t st, bool moments) {
   return dispatch(s, [&](auto lat, auto store, auto ft) {
     constexpr int Q = QOf<decltype(lat)>::Q;
-    return collide_stream_t<Q, decltype(store), decltype(ft)>(s, st);
+    return collide_stream_t<Q, decltype(store), decltype(ft)>(s, st, moments);
   });
 }
 

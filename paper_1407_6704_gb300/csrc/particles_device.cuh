@@ -510,19 +510,40 @@ __device__ __forceinline__ void sum_moments(const typename St::T (&v)[Q], typena
                                             typename St::R (&j)[3]) {
   using L = Lattice<Q>;
   using R = typename St::R;
-  R s = R(0), m0 = R(0), m1 = R(0), m2 = R(0);
+  if constexpr (sizeof(typename St::T) >= 4) {
+    // by opposite pairs: 16 additions instead of 21 in 2D, 39 instead of 49 in D3Q19
+    R s = St::load(v[0]);
+    bool any[3] = {false, false, false};
+    j[0] = j[1] = j[2] = R(0);
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    const R x = St::load(v[a]);
-    s += x;
-    if (L::e(a, 0)) m0 += L::e(a, 0) * x;
-    if (L::e(a, 1)) m1 += L::e(a, 1) * x;
-    if (L::e(a, 2)) m2 += L::e(a, 2) * x;
+    for (int a = 1; a < Q; a += 2) {
+      const R x0 = St::load(v[a]), x1 = St::load(v[a + 1]);
+      s += x0 + x1;
+      const R m = x0 - x1;
+#pragma unroll
+      for (int k = 0; k < L::D; ++k) {
+        if (L::e(a, k) == 0) continue;
+        j[k] = !any[k] ? (L::e(a, k) > 0 ? m : -m) : (L::e(a, k) > 0 ? j[k] + m : j[k] - m);
+        any[k] = true;
+      }
+    }
+    r = s;
+  } else {
+    // 16-bit storage keeps its order (see collide_cell_pairwise)
+    R s = R(0), m0 = R(0), m1 = R(0), m2 = R(0);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      const R x = St::load(v[a]);
+      s += x;
+      if (L::e(a, 0)) m0 += L::e(a, 0) * x;
+      if (L::e(a, 1)) m1 += L::e(a, 1) * x;
+      if (L::e(a, 2)) m2 += L::e(a, 2) * x;
+    }
+    r = s;
+    j[0] = m0;
+    j[1] = m1;
+    j[2] = m2;
   }
-  r = s;
-  j[0] = m0;
-  j[1] = m1;
-  j[2] = m2;
 }
 
 struct CoupleArgs {

@@ -587,8 +587,10 @@ __device__ __forceinline__ void axis_taps_local(int c, float f, int n, int perio
 // Launchers (defined in lbm.cu, particles.cu, reduce.cu)
 // ---------------------------------------------------------------------------
 // Fluid: one fused pull-stream + Guo-forced BGK collision, f[cur] -> f[1-cur];
-// consumes F and leaves it zero.
-cudaError_t launch_collide_stream(const State& s, cudaStream_t st);
+// consumes F and leaves it zero. moments: the moment field and the tile flags are those
+// of f[cur] (the particle phase of this step has run); FP64 storage then takes the
+// moments of busy cells from the field.
+cudaError_t launch_collide_stream(const State& s, cudaStream_t st, bool moments);
 // True when the collide-stream runs the two-cells-per-thread 16-bit kernel
 // (its block is 32 wide); the autotuner picks only the block height then.
 bool collide_uses_pair_kernel(const State& s);
