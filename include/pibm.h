@@ -89,7 +89,8 @@ extern "C" {
                                    the domain next to a wall; spreading keeps delta_width */
 
 /* scheduling of a step (results are the same either way) */
-#define PIBM_OVERLAP_AUTO 0 /* on for 2D lattices of at least 2^20 cells where supported */
+#define PIBM_OVERLAP_AUTO 0 /* 2D lattices of at least 2^20 cells, where supported: on with
+                               64-bit storage, the contact search alone with 32-bit storage */
 #define PIBM_OVERLAP_ON 1   /* on wherever supported */
 #define PIBM_OVERLAP_OFF 2  /* one stream, one collision kernel over the whole lattice */
 

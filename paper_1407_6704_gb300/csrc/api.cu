@@ -32,7 +32,7 @@ struct pibm_t {
   int64_t nstep;           // steps taken so far (any path)
   int64_t graph_kernels;   // kernels in one replay of the step graphs
   int graph_steps;         // steps in one replay of the step graphs
-  // overlap: contacts and the free tiles' collision on a second stream
+  // overlap: contacts (and the free tiles' collision) on a second stream
   int split;
   cudaStream_t side;
   cudaEvent_t ev_fork, ev_contacts, ev_free;
@@ -40,6 +40,13 @@ struct pibm_t {
 };
 
 namespace {
+
+// What a step runs on the handle's second stream.
+enum : int {
+  SPLIT_NONE = 0,
+  SPLIT_TILES = 1,     // contacts, then the free tiles' collision
+  SPLIT_CONTACTS = 2,  // contacts only
+};
 
 constexpr size_t ALIGN = 256;
 
@@ -249,7 +256,16 @@ int enqueue_step(pibm_t* h, cudaStream_t st, int* nk_out, bool split_ok = true) 
   // between rebuilds the storage order holds, so from the second step after a
   // rebuild the other buffer already holds the constants in that order
   s.move_consts = h->since_rebin <= 1;
-  if (h->split && split_ok) {
+  if (h->split == SPLIT_CONTACTS && split_ok) {
+    // side stream: contacts, beside the moments; the particle kernels wait for both
+    CK(cudaEventRecord(h->ev_fork, st));
+    CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+    PHASE(launch_contacts(s, h->side, &nk));
+    CK(cudaEventRecord(h->ev_contacts, h->side));
+    PHASE(launch_couple(s, st, &nk, h->ev_contacts));
+    PHASE(launch_collide_stream(s, st, true));
+    nk += 1;
+  } else if (h->split == SPLIT_TILES && split_ok) {
     // side stream: contacts, then the collision of the free tiles (no particle
     // stencil reaches them, so their force is zero and stays untouched); main
     // stream: moments, the particle kernels after the contacts, then the busy
@@ -625,12 +641,23 @@ int pibm_create(const pibm_config* cfg, void* workspace, size_t workspace_bytes,
     const int S = s.phy.substeps, det = s.deterministic;
     h->kernels_per_step = np == 0 ? 1 : (S <= 1 ? (det ? 13 : 11) : (det ? 12 : 11) + 2 * S);
   }
-  // overlap: a second stream and its events. AUTO takes it for 2D lattices of
-  // 2^20 cells or more; in 3D the tile-shaped collision (16-cell rows) is slower
-  // than the plain kernel by more than the overlap gains.
-  if (np > 0 && !s.deterministic && collide_tiles_supported(s) &&
-      (cfg->overlap == PIBM_OVERLAP_ON ||
-       (cfg->overlap == PIBM_OVERLAP_AUTO && d == 2 && s.geo.ncell >= (1LL << 20)))) {
+  // overlap: a second stream and its events. AUTO takes it for 2D lattices of 2^20
+  // cells or more; in 3D the tile-shaped collision (16-cell rows) is slower than the
+  // plain kernel by more than the overlap gains. In FP64 the free tiles' collision,
+  // bound by the FP64 pipe, hides behind the coupling's memory accesses (2048^2: 938
+  // us/step against 1,006 with the contacts alone beside the moments, 1,011 without);
+  // in FP32 both want the memory system, and one collision over the whole lattice after
+  // the coupling is faster (150.8 against 155.1 with and without the overlap). With
+  // sub-cycling the contacts belong to the sub-steps, so nothing is left to overlap.
+  int split = SPLIT_NONE;
+  if (np > 0 && !s.deterministic && collide_tiles_supported(s)) {
+    if (cfg->overlap == PIBM_OVERLAP_ON)
+      split = SPLIT_TILES;
+    else if (cfg->overlap == PIBM_OVERLAP_AUTO && d == 2 && s.geo.ncell >= (1LL << 20))
+      split = cfg->precision == PIBM_FP64 ? SPLIT_TILES
+                                          : (s.phy.substeps <= 1 ? SPLIT_CONTACTS : SPLIT_NONE);
+  }
+  if (split != SPLIT_NONE) {
     int lo = 0, hi = 0, sms = 0;
     if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
         cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, lo) != cudaSuccess ||
@@ -640,8 +667,8 @@ int pibm_create(const pibm_config* cfg, void* workspace, size_t workspace_bytes,
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
       return fail(PIBM_ECUDA);
     h->side_grid = 4 * sms;  // a share of the GPU beside the coupling kernels
-    h->split = 1;
-    h->kernels_per_step += 1;
+    h->split = split;
+    if (split == SPLIT_TILES) h->kernels_per_step += 1;
   }
   *out = h;
   return PIBM_OK;
