@@ -114,11 +114,13 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     // 32- and 16-bit storage: the particle update in FP64 (P64) or FP32
     constexpr bool NARROW = sizeof(R) == 4;
     // a warp takes 32 particles, or one round of it (8 four-point stencils, 16
-    // two-point ones) where 32 would leave an SM with less than one warp: the gathers
-    // of a particle then wait for no other round. 2D FP64 follows one rule at any
+    // two-point ones) where 32 would leave an SM with fewer than four warps: the gathers
+    // of a particle then wait for no other round (509 x 317 with 6,000 particles: 8.5 us
+    // at 32, 6.6 at 8; the update's FP64 work on a quarter of the lanes costs more once
+    // an SM has warps to switch between). 2D FP64 follows one rule at any
     // count: an ensemble member equals the same simulation stepped alone bit for bit.
     constexpr int PPW_FEW = W == 4 ? 8 : 16;
-    const bool few = P.np <= 152 * 32 && (D == 3 || COUPLE_BY_WARP<R>);
+    const bool few = P.np <= 4 * 152 * 32 && (D == 3 || COUPLE_BY_WARP<R>);
     auto couple = [&](auto kern, int ppw) {
       const unsigned w = warps_per_cta((P.np + ppw - 1) / ppw);
       static_assert(COUPLE_WARPS == 8, "warps_per_cta's largest");

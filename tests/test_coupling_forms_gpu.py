@@ -1,7 +1,7 @@
 """The forms of the particle coupling against one another: FP32 shares a particle's
 stencil among lanes (a warp takes 32 particles, or 8 or 16 where there are few), FP64
 keeps it on one lane except for few particles in 3D, and FP32 in 3D goes by tiles. Counts
-around a warp and around the switch (152 * 32), one particle and a ragged tail."""
+around a warp and around the switch (4 * 152 * 32), one particle and a ragged tail."""
 import numpy as np
 import pytest
 
@@ -21,6 +21,19 @@ pytestmark = pytest.mark.gpu
                           ("d3q15", (18, 19, 17), (0, 1, 0), 4, "lagrange4"),
                           ("d3q15", (18, 19, 17), (0, 0, 0), 2, "delta")])
 def test_fp32_forms_follow_fp64(lattice, n, periodic, width, interp, count):
+    check_forms(lattice, n, periodic, width, interp, count)
+
+
+@pytest.mark.parametrize("count", [19456, 19457])
+@pytest.mark.parametrize("lattice,n,periodic,width,interp",
+                         [("d2q9", (141, 133), (0, 1), 4, "delta"), ("d2q9", (141, 133), (0, 0), 2, "lagrange4"),
+                          ("d3q19", (36, 38, 33), (1, 0, 0), 4, "delta"),
+                          ("d3q15", (36, 38, 33), (0, 0, 1), 2, "lagrange4")])
+def test_fp32_forms_at_the_switch(lattice, n, periodic, width, interp, count):
+    check_forms(lattice, n, periodic, width, interp, count)
+
+
+def check_forms(lattice, n, periodic, width, interp, count):
     d = len(n)
     rng = np.random.default_rng(count)
     X = rng.uniform(0.1, np.array(n) - 0.1, (count, d))
