@@ -175,8 +175,9 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
       if constexpr (D == 3) {
         using S = StripShape<W, RE>;
         if (strips_fit<W, RE>(s.geo)) {
-          static_assert(S::PER_TILE == S::WARPS, "one CTA per tile");
-          k_spread_strips<W, RE, FT><<<(unsigned)ntiles, S::WARPS * 32, 0, st>>>(
+          static_assert(S::PER_TILE % S::WARPS == 0, "whole CTAs per tile");
+          k_spread_strips<W, RE, FT>
+              <<<(unsigned)(ntiles * (S::PER_TILE / S::WARPS)), S::WARPS * 32, 0, st>>>(
               s.geo, P.bm, P.np, P.tbusy, P.tn, P.tf, (const FT*)P.tr, P.bin_cnt, (FT*)s.F,
               s.err);
           return;

@@ -2230,10 +2230,10 @@ __device__ __forceinline__ void spread_gather_at(const Geometry& g, const BinMap
           }
           if (!in) continue;
           const FT* r = tr + (long long)sl * TAP_RECORD;
-          FT wt = r[o[0]] * r[4 + o[1]];
-          if constexpr (D == 3) wt *= r[8 + o[2]];
+          const FT wt = r[o[0]] * r[4 + o[1]];
 #pragma unroll
-          for (int k = 0; k < D; ++k) acc[k] = fma(r[12 + k], wt, acc[k]);
+          for (int k = 0; k < D; ++k)
+            acc[k] = fma(D == 3 ? r[12 + k] * r[8 + o[2]] : r[12 + k], wt, acc[k]);
         }
       }
     }
@@ -2263,8 +2263,10 @@ __global__ void __launch_bounds__(TileDims<D>::TC) k_spread_gather(
 // its terms in the same order and arithmetic as from spread_gather_at, so the results
 // are equal bit for bit. Each record is read once per strip instead of once per cell (in
 // the per-cell form half of the visits miss and the lanes of a warp read different
-// records). On a 64^3 lattice with 62,500 particles in FP64 407 -> 254 us, on 96^3 with
-// 20,000 196 -> 57 us. In 2D a cell has few visitors and the strips' serial walk costs
+// records). On a 64^3 lattice with 62,500 particles in FP64 407 -> 254 us, and 171 with
+// the cells' particles numbered through (a run of cells holds a few, and testing each
+// run's on its own left most lanes idle); on 96^3 with 20,000 196 -> 57 -> 45 us. One
+// strip a CTA: 175 us. Bound by the latency of its dependent steps. In 2D a cell has few visitors and the strips' serial walk costs
 // more (72 x 60: 9.6 us against 5.9).
 template <int W, int R, typename FT>
 __global__ void __launch_bounds__(StripShape<W, R>::WARPS * 32) k_spread_strips(
@@ -2272,13 +2274,13 @@ __global__ void __launch_bounds__(StripShape<W, R>::WARPS * 32) k_spread_strips(
     const unsigned* __restrict__ tn, const int4* __restrict__ tf, const FT* __restrict__ tr,
     const unsigned* __restrict__ start, FT* __restrict__ F, unsigned* __restrict__ err) {
   using S = StripShape<W, R>;
-  __shared__ FT acc_[S::WARPS][3][S::CELLS];
+  __shared__ FT acc_[S::WARPS][3][S::CELLS], qv[S::WARPS][S::QUEUE][3];
   __shared__ int2 queue[S::WARPS][S::QUEUE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Strip st = strip_of<W, R>(g, bm, tbusy, tn[0], blockIdx.x * S::WARPS + warp);
   if (!st.valid) return;  // the whole warp; no block-wide barrier below
   FT(&acc)[3][S::CELLS] = acc_[warp];
-  strip_sums<W, R, FT>(g, bm, np, st, tf, tr, start, err, acc, queue[warp]);
+  strip_sums<W, R, FT>(g, bm, np, st, tf, tr, start, err, acc, queue[warp], qv[warp]);
   for (int i = lane; i < S::CELLS; i += 32) {
     const int x = st.x0 + i % S::SX, y = st.y0 + i / S::SX;
     if (x >= g.n[0] || y >= g.n[1]) continue;

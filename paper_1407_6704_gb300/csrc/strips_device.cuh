@@ -8,15 +8,16 @@ namespace pibm {
 
 namespace {
 
-// A warp owns a strip of 128 cells: one z plane of a busy tile.
+// A warp owns a strip of 128 cells: one z plane of a busy tile; the strips of a tile
+// share a CTA, and so the records in its L1.
 template <int W, int R>
 struct StripShape {
   using TD = TileDims<3>;
   static constexpr int SX = TD::TX, SY = TD::TY;
   static constexpr int CELLS = SX * SY;
   static constexpr int PER_TILE = TD::TC / CELLS;
-  static constexpr int WARPS = 4;  // per CTA
-  static constexpr int QUEUE = 128;
+  static constexpr int QUEUE = 64;
+  static constexpr int WARPS = 4;  // strips per CTA
   static constexpr int ROWS = (SY + 2 * R) * (2 * R + 1);
   static constexpr int SEGS = ROWS * (2 * R + 1);  // R single cells, the strip's run, R cells
 };
@@ -68,7 +69,8 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
                                            const FT* __restrict__ tr,
                                            const unsigned* __restrict__ start, unsigned* err,
                                            FT (&acc)[3][StripShape<W, R>::CELLS],
-                                           int2 (&queue)[StripShape<W, R>::QUEUE]) {
+                                           int2 (&queue)[StripShape<W, R>::QUEUE],
+                                           FT (&qv)[StripShape<W, R>::QUEUE][3]) {
   using S = StripShape<W, R>;
   constexpr int NODES = W * W, CPL = 32 / NODES;  // components side by side in a warp
   constexpr int NC = 3, TURNS = (NC + CPL - 1) / CPL;
@@ -100,10 +102,10 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
         const int rx = (e.y & 0xff) - 8 + ni, ry = ((e.y >> 8) & 0xff) - 8 + nj;
         in[u] = rx >= 0 && rx < S::SX && ry >= 0 && ry < S::SY;
         c[u] = ry * S::SX + rx;
-        wt[u] = r[ni] * r[4 + nj] * r[8 + (e.y >> 16)];
+        wt[u] = r[ni] * r[4 + nj];
 #pragma unroll
         for (int t = 0; t < TURNS; ++t)
-          if (comp + t * CPL < NC) v[u][t] = r[12 + comp + t * CPL];
+          if (comp + t * CPL < NC) v[u][t] = qv[i0 + u][comp + t * CPL];
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -141,39 +143,63 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
       atomicOr(err, ERR_INDEX);
       hi = lo = 0;
     }
-    unsigned some = __ballot_sync(0xffffffffu, hi > lo);
-    while (some) {
-      const int src = __ffs(some) - 1;
-      some &= some - 1;
-      const unsigned a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
-      for (unsigned p0 = a; p0 < b; p0 += 32) {
-        const unsigned sl = p0 + lane;
-        bool hit = false;
-        int word = 0;
-        if (sl < b) {
-          const int4 f = tf[sl];
-          // first node relative to the strip, in the image that can reach it
-          int dx = f.x - st.x0, dy = f.y - st.y0, dz = st.z0 - f.z;
-          if (g.periodic[0]) {
-            if (dx <= S::SX - g.n[0]) dx += g.n[0];
-            else if (dx >= g.n[0] - W) dx -= g.n[0];
-          }
-          if (g.periodic[1]) {
-            if (dy <= S::SY - g.n[1]) dy += g.n[1];
-            else if (dy >= g.n[1] - W) dy -= g.n[1];
-          }
-          if (g.periodic[2]) {
-            if (dz < 0) dz += g.n[2];
-            else if (dz >= g.n[2]) dz -= g.n[2];
-          }
-          hit = dx > -W && dx < S::SX && dy > -W && dy < S::SY && dz >= 0 && dz < W;
-          word = hit ? (dx + 8) | (dy + 8) << 8 | dz << 16 : 0;
-        }
-        const unsigned hits = __ballot_sync(0xffffffffu, hit);
-        if (queued + __popc(hits) > S::QUEUE) drain();
-        if (hit) queue[queued + __popc(hits & ((1u << lane) - 1u))] = make_int2((int)sl, word);
-        queued += __popc(hits);
+    // the particles of the 32 segments in order, 32 at a time: lane l of a turn takes
+    // particle base + l, in the segment whose range of running counts holds it
+    unsigned incl = hi - lo;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned before = lo - (incl - (hi - lo));  // slot = before + running index
+    for (unsigned base = 0; base < total; base += 32) {
+      const unsigned idx = base + lane;
+      int seg = 0;  // segments whose particles all come before idx
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned u = __shfl_sync(0xffffffffu, incl, seg + o - 1);
+        if (u <= idx) seg += o;
       }
+      const unsigned sl = __shfl_sync(0xffffffffu, before, seg & 31) + idx;
+      bool hit = false;
+      int word = 0;
+      FT v[3] = {FT(0), FT(0), FT(0)};
+      if (idx < total) {
+        const int4 f = tf[sl];
+        // first node relative to the strip, in the image that can reach it
+        int dx = f.x - st.x0, dy = f.y - st.y0, dz = st.z0 - f.z;
+        if (g.periodic[0]) {
+          if (dx <= S::SX - g.n[0]) dx += g.n[0];
+          else if (dx >= g.n[0] - W) dx -= g.n[0];
+        }
+        if (g.periodic[1]) {
+          if (dy <= S::SY - g.n[1]) dy += g.n[1];
+          else if (dy >= g.n[1] - W) dy -= g.n[1];
+        }
+        if (g.periodic[2]) {
+          if (dz < 0) dz += g.n[2];
+          else if (dz >= g.n[2]) dz -= g.n[2];
+        }
+        hit = dx > -W && dx < S::SX && dy > -W && dy < S::SY && dz >= 0 && dz < W;
+        if (hit) {
+          // A_p g times the weight of the strip's plane, once per particle
+          word = (dx + 8) | (dy + 8) << 8;
+          const FT* r = tr + (long long)sl * TAP_RECORD;
+          const FT wz = r[8 + dz];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) v[k] = r[12 + k] * wz;
+        }
+      }
+      const unsigned hits = __ballot_sync(0xffffffffu, hit);
+      if (queued + __popc(hits) > S::QUEUE) drain();
+      if (hit) {
+        const int i = queued + __popc(hits & ((1u << lane) - 1u));
+        queue[i] = make_int2((int)sl, word);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) qv[i][k] = v[k];
+      }
+      queued += __popc(hits);
     }
   }
   drain();
