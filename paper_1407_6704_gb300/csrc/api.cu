@@ -1,10 +1,14 @@
 // Host side of the C ABI declared in include/pibm.h: validation, workspace
 // layout, upload of the initial state, the step loop (replayed from CUDA graphs
 // of two steps) and the read-back calls.
+#include <errno.h>
 #include <math.h>
+#include <stdint.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <new>
@@ -51,6 +55,25 @@ enum : int {
 constexpr size_t ALIGN = 256;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
+
+// Map the pages of a host array that a copy is about to fill (its contents stay). Into
+// pages that no one has touched the device writes at 1 to 4 GB/s, one page fault after
+// another; mapped ones take 100 GB/s, and the host maps 30 GB/s, while queued steps still
+// run if there are any. A read into new arrays of 15 MB: 8.4 -> 0.73 ms, of 100 MB: 26 ->
+// 4.6 ms, on an idle device. Below 1 MiB allocators return memory in use. Where the
+// kernel or the memory does not support it (pinned memory), nothing happens.
+void map_pages(void* dst, size_t bytes) {
+#ifdef MADV_POPULATE_WRITE
+  if (bytes < (size_t(1) << 20)) return;
+  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+  const uintptr_t lo = (uintptr_t)dst / page * page;
+  const int keep = errno;
+  (void)madvise((void*)lo, (uintptr_t)dst + bytes - lo, MADV_POPULATE_WRITE);
+  errno = keep;
+#else
+  (void)dst, (void)bytes;
+#endif
+}
 
 struct Layout {
   size_t f, F, mom, red, err, out, X, U, rad, mass, Ap, buoy, gw, cf, pid, rl, jl, Fs, tf, tr, nb, nbn, xs0, xr, cr, xs, cs, g, Fc, Fcf, key, rank, perm, bin,
@@ -746,6 +769,11 @@ int pibm_read_fields(pibm_t* h, unsigned mask, void* const* dst, int on_device) 
   if (on_device) {
     if (rho || mom || pop) CK(launch_read_state(s, rho, mom, pop, 0, pop ? q : 0, st));
   } else {
+    const size_t bytes[PIBM_NFIELDS] = {sizeof(double) * nc, sizeof(double) * nc * d,
+                                        sizeof(double) * nc * q, sizeof(double) * d * np,
+                                        sizeof(double) * d * np};
+    for (int k = 0; k < PIBM_NFIELDS; ++k)
+      if (mask >> k & 1u) map_pages(dst[k], bytes[k]);
     // as many planes per launch as the stage holds (rho, the d planes of j and the
     // population planes, in this order); the copies follow their kernel on the
     // stream, and the next launch follows them

@@ -77,3 +77,34 @@ def test_particles_come_back_in_user_order(n, count):
     assert np.array_equal(sim.read("x")["x"], r["x"])
     assert np.array_equal(sim.read("u")["u"], r["u"])
     sim.close()
+
+
+@pytest.mark.parametrize("n", [(120, 121), (300, 301)])
+def test_large_host_arrays(n):
+    """Arrays above a megabyte, which are mapped before the copy: new, in use, pinned, and
+    not starting on a page."""
+    import torch
+
+    count = 40000 * (n[0] > 200) + 50
+    rng = np.random.default_rng(2)
+    sim = Pibm("d2q9", n, (1, 0), 0.8, kn=0.0, x0=rng.uniform(0.5, np.array(n) - 0.5, (count, 2)),
+               u0=inputs.velocities(count, 2, seed=6, scale=1e-6), diameter=np.full(count, 0.1),
+               density_ratio=np.full(count, 2.0))
+    names = ("rho", "j", "pop", "x", "u")
+    sim.step(3)
+    r = sim.read(*names)
+    shapes = {k: r[k].shape for k in names}
+    pinned = {k: torch.full(shapes[k], -1.0, dtype=torch.float64, pin_memory=True).numpy()
+              for k in names}
+    shifted = {}
+    for k in names:
+        raw = np.full(r[k].size + 3, -1.0)
+        shifted[k] = raw[1:-2].reshape(shapes[k])
+    for out in (pinned, shifted):
+        got = sim.read(*names, out=out)
+        for k in names:
+            assert np.array_equal(got[k], r[k]) and np.shares_memory(got[k], out[k])
+    for k in names:
+        raw = shifted[k].base if shifted[k].base.ndim == 1 else shifted[k].base.base
+        assert raw[0] == -1.0 and (raw[-2:] == -1.0).all()
+    sim.close()
