@@ -182,7 +182,7 @@ def collide_fp64_ops(q):
         pc = ent["per_cell"]
         fl, ins, src = pc["flops"], pc["instructions"], "ncu instruction counts"
     except Exception:
-        fl, ins, src = 136, 95, "estimate"
+        fl, ins, src = 91, 63, "estimate"
     if q != 9:
         fl, ins, src = fl * q / 9.0, ins * q / 9.0, "D2Q9 counts scaled by q/9 (estimate)"
     ceiling = 2.0 * (fl / ins) * 152 * 2.07e9 / 1e12
@@ -394,8 +394,8 @@ def run_gpu(args, rank, world):
                    "parallelism": f"replicas x{world}",
                    "cell_list_rebuild_every": args.rebin,
                    "warmup_steps_run": warmup_steps(args),
-                   "overlap": "auto: on for this 2D lattice (contacts and the particle-free "
-                              "tiles' collision on a second stream)",
+                   "overlap": "auto: the contact search on a second stream (with 64-bit "
+                              "storage the particle-free tiles' collision as well)",
                    "l2": "inputs larger than L2 (population buffers 2x151 MB f32 / 2x302 MB f64)"},
         "phases_ms_per_step": ph,
         "kernels": kern,
