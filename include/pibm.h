@@ -238,7 +238,7 @@ int pibm_status(pibm_t* h);
 
 /* Number of kernels one pibm_step(h, 1) launches (for launch accounting); with
  * rebin_every > 1, the count of a step that rebuilds the cell list. With
- * overlap the collision counts as two kernels (free and busy tiles). */
+ * the free tiles' collision on the second stream the collision counts as two kernels. */
 int pibm_kernels_per_step(pibm_t* h);
 
 /* Total number of kernels pibm_step has launched on this handle since it was

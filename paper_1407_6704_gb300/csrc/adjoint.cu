@@ -1050,9 +1050,9 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
     return cudaSuccess;
   };
   // Full stretches recur with the same arguments (up to the buffer parity they start
-  // from), so from the fourth stretch on they are captured once and replayed: a step of a
-  // small lattice is 13 launches of a few microseconds each, and launching them one by
-  // one took longer than running them (72 x 60, 120 steps: 23.3 ms for 14.9 ms of
+  // from), so in runs of four stretches or more they are captured once and replayed: a
+  // step of a small lattice is 13 launches of a few microseconds each, and launching them
+  // one by one took longer than running them (72 x 60, 120 steps: 23.3 ms for 14.9 ms of
   // kernels).
   StretchGraphs graphs;
   bool replayed = grads && nseg >= 4 && K <= 64 &&
