@@ -74,13 +74,15 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   constexpr int D = Lattice<Q>::D;
   using T = typename St::T;
   using R = typename St::R;
-  // the particle kernels see the dimension and the arithmetic type only: one
-  // instantiation serves every velocity set and storage type of them
+  // the particle kernels see the dimension, the arithmetic type and whether sums keep
+  // their order (16-bit storage): one instantiation serves every velocity set and both
+  // 16-bit types; the tile kernel adds in that order in any storage
   constexpr int QC = D == 2 ? 9 : 19;
-  using SC = typename std::conditional<sizeof(R) == 8, StoreF64, StoreF32>::type;
+  using SA = typename std::conditional<sizeof(R) == 8, StoreF64, StoreF32>::type;
+  using SC = typename std::conditional<IN_ORDER<St>, StoreF16, SA>::type;
   CoupleArgs A = couple_args(s);
   const long long ntiles = P.nbin / P.bm.tc;
-  const unsigned pt = particle_threads(P.np), pb = blocks_for(P.np, pt);
+  const unsigned pt = IN_ORDER<St> ? 256 : particle_threads(P.np), pb = blocks_for(P.np, pt);
   auto moments = [&](auto threads) {
     constexpr int TH = decltype(threads)::value;
     using Sh = MomentsShape<Q, St, TH>;
@@ -106,8 +108,8 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
         constexpr int TPC = CoupleWindow<D, W>::TPC;
         const long long groups = (P.ntiles + TPC - 1) / TPC;
         const unsigned grid = (unsigned)(groups * TILE_CHUNKS);
-        if (s.phy.p64) k_couple_tiles<QC, W, SC, FT, true><<<grid, 256, 0, st>>>(A);
-        else k_couple_tiles<QC, W, SC, FT, false><<<grid, 256, 0, st>>>(A);
+        if (s.phy.p64) k_couple_tiles<QC, W, SA, FT, true><<<grid, 256, 0, st>>>(A);
+        else k_couple_tiles<QC, W, SA, FT, false><<<grid, 256, 0, st>>>(A);
         tiled = true;
       }
     }
@@ -119,10 +121,12 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     // at 32, 6.6 at 8; the update's FP64 work on a quarter of the lanes costs more once
     // an SM has warps to switch between). 2D FP64 follows one rule at any
     // count: an ensemble member equals the same simulation stepped alone bit for bit.
+    // 16-bit storage keeps whole warps in CTAs of 256 threads (IN_ORDER).
     constexpr int PPW_FEW = W == 4 ? 8 : 16;
-    const bool few = P.np <= 4 * 152 * 32 && (D == 3 || COUPLE_BY_WARP<R>);
+    const bool few =
+        P.np <= 4 * 152 * 32 && (COUPLE_BY_WARP<SC> || (D == 3 && !IN_ORDER<SC>));
     auto couple = [&](auto kern, int ppw) {
-      const unsigned w = warps_per_cta((P.np + ppw - 1) / ppw);
+      const unsigned w = IN_ORDER<SC> ? COUPLE_WARPS : warps_per_cta((P.np + ppw - 1) / ppw);
       static_assert(COUPLE_WARPS == 8, "warps_per_cta's largest");
       kern<<<blocks_for(P.np, w * ppw), w * 32, 0, st>>>(A);
     };

@@ -1165,8 +1165,34 @@ __device__ __forceinline__ void gather_moments(const CoupleArgs& A, const Taps<W
   }
 }
 
+// One row of a 2D FP32 stencil whose W cells are consecutive (no wall drop, no
+// wrap): the force of two neighbouring cells (Fx, Fy, Fx, Fy) is one 16-byte
+// vector atomic when the first of them has an even index, so a row takes W/2
+// atomics (aligned) or W/2 + 1 (one lone cell at each end), and so fewer L1
+// sector requests than one atomic per cell.
+template <int W>
+__device__ __forceinline__ void spread_row_pairs(float* __restrict__ F, long long c0,
+                                                 const float (&wt)[W], float ax, float ay) {
+  float2* F2 = reinterpret_cast<float2*>(F);
+  float4* F4 = reinterpret_cast<float4*>(F);
+  int i = 0;
+  if (c0 & 1) {
+    atomicAdd(F2 + c0, make_float2(ax * wt[0], ay * wt[0]));
+    i = 1;
+  }
+#pragma unroll
+  for (int k = 0; k < W / 2; ++k) {
+    const int j = i + 2 * k;
+    if (j + 1 < W)
+      atomicAdd(F4 + ((c0 + j) >> 1),
+                make_float4(ax * wt[j], ay * wt[j], ax * wt[j + 1], ay * wt[j + 1]));
+  }
+  if (c0 & 1) atomicAdd(F2 + c0 + W - 1, make_float2(ax * wt[W - 1], ay * wt[W - 1]));
+}
+
 // Eq. (9): add amp * w to F at every tap (one vector atomic per cell in FP32,
-// one atomic per component in FP64).
+// one atomic per component in FP64; in 2D FP32, rows of consecutive cells by
+// pairs of cells).
 template <int D, int W, typename TW, typename FT>
 __device__ __forceinline__ void spread_amp(const CoupleArgs& A, const Taps<W, TW>& tx,
                                            const Taps<W, TW>& ty, const Taps<W, TW>& tz,
@@ -1174,6 +1200,21 @@ __device__ __forceinline__ void spread_amp(const CoupleArgs& A, const Taps<W, TW
   constexpr int WZ = D == 3 ? W : 1;
   const Geometry& g = A.g;
   FT* F = (FT*)A.F;
+  if constexpr (D == 2 && sizeof(FT) == 4) {
+    if (tx.idx[W - 1] == tx.idx[0] + (W - 1)) {  // consecutive: no dropped node, no wrap
+#pragma unroll
+      for (int iy = 0; iy < W; ++iy) {
+        const FT wyz = (FT)ty.w[iy];
+        if (wyz == FT(0)) continue;
+        float wt[W];
+#pragma unroll
+        for (int ix = 0; ix < W; ++ix) wt[ix] = (FT)tx.w[ix] * wyz;
+        spread_row_pairs<W>((float*)F, (long long)ty.idx[iy] * g.n[0] + tx.idx[0], wt, amp[0],
+                            amp[1]);
+      }
+      return;
+    }
+  }
 #pragma unroll 1
   for (int iz = 0; iz < WZ; ++iz) {
     FT wz = FT(1);
@@ -1197,6 +1238,24 @@ __device__ __forceinline__ void spread_amp(const CoupleArgs& A, const Taps<W, TW
     }
   }
 }
+
+// 16-bit storage: one lane gathers and spreads the whole stencil of a particle, in 2D and
+// wherever the tile kernel (which adds in the same order) does not take it. FP32 sums and
+// products in another order, or atomics of the lanes interleaved in another way, differ by
+// FP32 rounding, and 16-bit storage turns that into other stored values: with the stencils
+// shared out among lanes the particle velocities were 1e-5 to 6e-4 of their norm away
+// after 50 steps, at the same error against 64 bits. A run of 2048^2 with 500,000
+// particles in FP16 takes 3.38 ms per 20 steps and read-back, 3.11 with shared stencils.
+template <class St>
+constexpr bool IN_ORDER = sizeof(typename St::T) == 2;
+
+// Whether the coupling shares a particle's stencil among lanes (couple_warp) or keeps
+// it on one (couple_at). In FP32 sharing halves the sectors; in FP64 the FP64 pipe
+// bounds either form, the shared one adds the lanes' partial sums on top, and the
+// moments are two sectors per cell anyway: 62,500 particles of a 64^3 lattice take
+// 123 us shared and 88 us on one lane each, 500,000 in 2D step in 972 and 954 us.
+template <class St>
+constexpr bool COUPLE_BY_WARP = sizeof(typename St::R) == 4 && !IN_ORDER<St>;
 
 // --- one warp, 32 particles: the stencils shared out by cells -----------------
 // Every lane owns a particle (record, taps, update); the gathers and the spreading
@@ -1658,12 +1717,14 @@ __device__ __forceinline__ void couple_warp(const CoupleArgs& A, long long sl0,
   }
 }
 
-// The same with one thread per particle, in FP64: every tap of the stencil is gathered
-// and spread by the particle's own lane, with the taps in registers.
+// The same with one thread per particle: every tap of the stencil is gathered and spread
+// by the particle's own lane, with the taps in registers. In FP32 arithmetic the taps of the
+// spreading come from a fresh read of the record (which the update's stores may alias): a
+// few FP32 operations, and the registers are the update's in between; the particle's state
+// is loaded after the gathers of a 2D stencil for the same reason.
 template <int Q, int W, class St, typename FT, bool LAG, bool NC, bool P64>
 __device__ __forceinline__ void couple_at(const CoupleArgs& A, long long sl) {
   using R = typename St::R;
-  static_assert(sizeof(R) == 8, "FP32 arithmetic goes by warps");
   constexpr int D = Lattice<Q>::D;
   constexpr int WI = LAG ? 4 : W;
   const Geometry& g = A.g;
@@ -1676,21 +1737,29 @@ __device__ __forceinline__ void couple_at(const CoupleArgs& A, long long sl) {
     atomicOr(A.err, ERR_INDEX);
     return;
   }
-  double X[3] = {0.0, 0.0, 0.0}, U[3] = {0.0, 0.0, 0.0}, Fc[3] = {0.0, 0.0, 0.0};
+  using FCT = typename std::conditional<sizeof(R) == 8 || P64, double, R>::type;
+  double X[3] = {0.0, 0.0, 0.0}, U[3] = {0.0, 0.0, 0.0};
+  FCT Fc[3] = {FCT(0), FCT(0), FCT(0)};
+  auto load_state = [&]() {
 #pragma unroll
-  for (int k = 0; k < D; ++k) {
-    X[k] = A.X[k * np + p];
-    U[k] = A.U[k * np + p];
-    Fc[k] = A.Fcout[k * np + sl];
-  }
+    for (int k = 0; k < D; ++k) {
+      X[k] = A.X[k * np + p];
+      U[k] = A.U[k * np + p];
+      if constexpr (sizeof(R) == 8 || P64) Fc[k] = A.Fcout[k * np + sl];
+      else Fc[k] = A.Fcf ? A.Fcf[k * np + sl] : (R)A.Fcout[k * np + sl];
+    }
+  };
+  constexpr bool LATE = D == 2 && sizeof(R) == 4;
+  if constexpr (!LATE) load_state();
   // --- interpolation of rho, j (Eq. 4) ---
   Taps<WI, R> tx, ty, tz;
   particle_taps<D, WI, LAG, R>(g, mc, mf, X, tx, ty, tz);
   R rs, js[3];
   gather_moments<D, WI, R, NC>(A, tx, ty, tz, rs, js);
+  if constexpr (LATE) load_state();
   // --- particle update (Eq. 13) and force density (Eqs. 6-7) ---
   FT amp[3] = {FT(0), FT(0), FT(0)};
-  advance_particle<D, St, FT, P64, double>(A, sl, p, mc, mf, X, U, Fc, rs, js, amp);
+  advance_particle<D, St, FT, P64, FCT>(A, sl, p, mc, mf, X, U, Fc, rs, js, amp);
   // --- spreading (Eq. 9) with the delta kernel ---
   auto spread = [&](const Taps<W, R>& sx, const Taps<W, R>& sy, const Taps<W, R>& sz) {
     if (A.spread) {
@@ -1700,28 +1769,21 @@ __device__ __forceinline__ void couple_at(const CoupleArgs& A, long long sl) {
       keep_amp<FT>(A, sl, amp);
     }
   };
-  if constexpr (LAG) {
+  if constexpr (LAG || sizeof(R) == 4) {
+    const float4 mf2 = A.xs[sl];
     Taps<W, R> sx, sy, sz;
-    particle_taps<D, W, false, R>(g, mc, mf, X, sx, sy, sz);
+    particle_taps<D, W, false, R>(g, mc, mf2, X, sx, sy, sz);
     spread(sx, sy, sz);
   } else {
     spread(tx, ty, tz);
   }
 }
 
-// Whether the coupling shares a particle's stencil among lanes (couple_warp) or keeps
-// it on one (couple_at). In FP32 sharing halves the sectors; in FP64 the FP64 pipe
-// bounds either form, the shared one adds the lanes' partial sums on top, and the
-// moments are two sectors per cell anyway: 62,500 particles of a 64^3 lattice take
-// 123 us shared and 88 us on one lane each, 500,000 in 2D step in 972 and 954 us.
-template <typename R>
-constexpr bool COUPLE_BY_WARP = sizeof(R) == 4;
-
 // The particles of the calling warp, 32 (or PPW) slots from sl0 on.
 template <int Q, int W, class St, typename FT, bool LAG, bool NC, bool P64, int PPW>
 __device__ __forceinline__ void couple_slots(const CoupleArgs& A, long long sl0,
                                              CoupleStage<Q, W, St, LAG>& stage) {
-  if constexpr (COUPLE_BY_WARP<typename St::R> || PPW < 32)
+  if constexpr (COUPLE_BY_WARP<St> || PPW < 32)
     couple_warp<Q, W, St, FT, LAG, NC, P64, PPW>(A, sl0, stage);
   else
     couple_at<Q, W, St, FT, LAG, NC, P64>(A, sl0 + (threadIdx.x & 31));
@@ -1732,7 +1794,10 @@ constexpr int COUPLE_WARPS = 8;
 
 template <int Q, int W, class St, typename FT, bool LAG, bool P64, int PPW>
 __global__ void __launch_bounds__(COUPLE_WARPS * 32,
-                                  sizeof(typename St::R) == 4 ? (Lattice<Q>::D == 2 ? 5 : 4) : 2)
+                                  sizeof(typename St::R) == 8 ? 2
+                                  : Lattice<Q>::D == 2        ? 5
+                                  : IN_ORDER<St>              ? 3   // at 4, 80 bytes spilt
+                                                              : 4)
     k_couple(CoupleArgs A) {
   __shared__ CoupleStage<Q, W, St, LAG> stage[COUPLE_WARPS];
   const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -2094,10 +2159,14 @@ __global__ void __launch_bounds__(COUPLE_WARPS * 32) k_sub_init(CoupleArgs A) {
       on = false;
     }
   }
-  stage_taps<D, WI, R>(stage, lane, on, tx, ty, tz);
-  __syncwarp();
-  R rs, js[3];
-  gather_warp<D, WI, R, true, WI>(A, stage, lane, rs, js);
+  R rs = R(0), js[3] = {R(0), R(0), R(0)};
+  if constexpr (IN_ORDER<St>) {
+    if (on) gather_moments<D, WI, R>(A, tx, ty, tz, rs, js);
+  } else {
+    stage_taps<D, WI, R>(stage, lane, on, tx, ty, tz);
+    __syncwarp();
+    gather_warp<D, WI, R, true, WI>(A, stage, lane, rs, js);
+  }
   if (!act) return;
   if (!A.spread) {  // ordered spreading at the end of the step: keep the taps
     Taps<W, R> sx, sy, sz;
@@ -2203,6 +2272,10 @@ __global__ void __launch_bounds__(COUPLE_WARPS * 32) k_sub_spread(CoupleArgs A) 
       particle_taps<D, W, false, R>(A.g, mc, mf, X, tx, ty, tz);
     }
   }
+  if constexpr (IN_ORDER<St>) {
+    if (act) spread_amp<D, W, R, FT>(A, tx, ty, tz, amp);
+    return;
+  }
   stage_taps<D, W, R>(stage, lane, act, tx, ty, tz);
 #pragma unroll
   for (int k = 0; k < 3; ++k) stage.amp[lane][k] = amp[k];
@@ -2275,10 +2348,10 @@ __device__ __forceinline__ void spread_gather_at(const Geometry& g, const BinMap
           }
           if (!in) continue;
           const FT* r = tr + (long long)sl * TAP_RECORD;
-          const FT wt = r[o[0]] * r[4 + o[1]];
+          FT wt = r[o[0]] * r[4 + o[1]], wa = FT(1);
+          if constexpr (D == 3) (PLANE_WITH_AMP<FT> ? wa : wt) *= r[8 + o[2]];
 #pragma unroll
-          for (int k = 0; k < D; ++k)
-            acc[k] = fma(D == 3 ? r[12 + k] * r[8 + o[2]] : r[12 + k], wt, acc[k]);
+          for (int k = 0; k < D; ++k) acc[k] = fma(r[12 + k] * wa, wt, acc[k]);
         }
       }
     }
@@ -2319,7 +2392,7 @@ __global__ void __launch_bounds__(StripShape<W, R>::WARPS * 32) k_spread_strips(
     const unsigned* __restrict__ tn, const int4* __restrict__ tf, const FT* __restrict__ tr,
     const unsigned* __restrict__ start, FT* __restrict__ F, unsigned* __restrict__ err) {
   using S = StripShape<W, R>;
-  __shared__ FT acc_[S::WARPS][3][S::CELLS], qv[S::WARPS][S::QUEUE][3];
+  __shared__ FT acc_[S::WARPS][3][S::CELLS], qv[S::WARPS][S::QUEUE][QUEUED<FT>];
   __shared__ int2 queue[S::WARPS][S::QUEUE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Strip st = strip_of<W, R>(g, bm, tbusy, tn[0], blockIdx.x * S::WARPS + warp);

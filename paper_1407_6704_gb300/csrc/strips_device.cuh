@@ -33,6 +33,17 @@ bool strips_fit(const Geometry& g) {
   return true;
 }
 
+// Where the weight wz of a term A_p g wx wy wz goes in the ordered sums. FP32 multiplies
+// the weights first, ((wx wy) wz) A_p g, as the atomic spreading does: 16-bit storage
+// turns another rounding into other stored values. FP64 multiplies A_p g once per particle
+// and plane instead of the weights once per node: slice of 64^3 with 62,500 particles,
+// 10 steps: 3.88 ms against 3.97.
+template <typename FT>
+constexpr bool PLANE_WITH_AMP = sizeof(FT) == 8;
+// Values queued per particle: A_p g, and wz where it goes with the weights.
+template <typename FT>
+constexpr int QUEUED = PLANE_WITH_AMP<FT> ? 3 : 4;
+
 // Where a strip lies; valid is false past the end of the list or of the lattice.
 struct Strip {
   int x0, y0, z0;
@@ -70,7 +81,7 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
                                            const unsigned* __restrict__ start, unsigned* err,
                                            FT (&acc)[3][StripShape<W, R>::CELLS],
                                            int2 (&queue)[StripShape<W, R>::QUEUE],
-                                           FT (&qv)[StripShape<W, R>::QUEUE][3]) {
+                                           FT (&qv)[StripShape<W, R>::QUEUE][QUEUED<FT>]) {
   using S = StripShape<W, R>;
   constexpr int NODES = W * W, CPL = 32 / NODES;  // components side by side in a warp
   constexpr int NC = 3, TURNS = (NC + CPL - 1) / CPL;
@@ -103,6 +114,7 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
         in[u] = rx >= 0 && rx < S::SX && ry >= 0 && ry < S::SY;
         c[u] = ry * S::SX + rx;
         wt[u] = r[ni] * r[4 + nj];
+        if constexpr (!PLANE_WITH_AMP<FT>) wt[u] *= qv[i0 + u][3];
 #pragma unroll
         for (int t = 0; t < TURNS; ++t)
           if (comp + t * CPL < NC) v[u][t] = qv[i0 + u][comp + t * CPL];
@@ -164,7 +176,7 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
       const unsigned sl = __shfl_sync(0xffffffffu, before, seg & 31) + idx;
       bool hit = false;
       int word = 0;
-      FT v[3] = {FT(0), FT(0), FT(0)};
+      FT v[QUEUED<FT>] = {};
       if (idx < total) {
         const int4 f = tf[sl];
         // first node relative to the strip, in the image that can reach it
@@ -183,12 +195,13 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
         }
         hit = dx > -W && dx < S::SX && dy > -W && dy < S::SY && dz >= 0 && dz < W;
         if (hit) {
-          // A_p g times the weight of the strip's plane, once per particle
+          // A_p g and the weight of the strip's plane, once per particle
           word = (dx + 8) | (dy + 8) << 8;
           const FT* r = tr + (long long)sl * TAP_RECORD;
           const FT wz = r[8 + dz];
 #pragma unroll
-          for (int k = 0; k < 3; ++k) v[k] = r[12 + k] * wz;
+          for (int k = 0; k < 3; ++k) v[k] = PLANE_WITH_AMP<FT> ? r[12 + k] * wz : r[12 + k];
+          if constexpr (!PLANE_WITH_AMP<FT>) v[3] = wz;
         }
       }
       const unsigned hits = __ballot_sync(0xffffffffu, hit);
@@ -197,7 +210,7 @@ __device__ __forceinline__ void strip_sums(const Geometry& g, const BinMap& bm, 
         const int i = queued + __popc(hits & ((1u << lane) - 1u));
         queue[i] = make_int2((int)sl, word);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) qv[i][k] = v[k];
+        for (int k = 0; k < QUEUED<FT>; ++k) qv[i][k] = v[k];
       }
       queued += __popc(hits);
     }
