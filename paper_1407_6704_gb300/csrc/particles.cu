@@ -150,7 +150,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   } else {
     // DEM sub-cycling: interpolate once, S x (contacts, update), then spread
     if (s.phy.lagrange)
-      k_sub_init<QC, 4, SC, true><<<pb, pt, 0, st>>>(A);
+      k_sub_init<QC, W, SC, true><<<pb, pt, 0, st>>>(A);
     else
       k_sub_init<QC, W, SC, false><<<pb, pt, 0, st>>>(A);
     const double h = 1.0 / (double)s.phy.substeps;
