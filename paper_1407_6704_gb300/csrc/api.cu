@@ -587,6 +587,8 @@ int pibm_create(const pibm_config* cfg, void* workspace, size_t workspace_bytes,
     pibm_destroy(h);
     return code;
   };
+  if (cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+    return fail(PIBM_ECUDA);
   // force field and health word start at zero
   if (cudaMemsetAsync(s.F, 0, (size_t)(d == 2 ? 2 : 4) * s.geo.pitch * fs, st) != cudaSuccess ||
       cudaMemsetAsync(s.err, 0, sizeof(unsigned), st) != cudaSuccess)
@@ -681,15 +683,14 @@ int pibm_create(const pibm_config* cfg, void* workspace, size_t workspace_bytes,
                                           : (s.phy.substeps <= 1 ? SPLIT_CONTACTS : SPLIT_NONE);
   }
   if (split != SPLIT_NONE) {
-    int lo = 0, hi = 0, sms = 0;
+    int lo = 0, hi = 0;
     if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
         cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, lo) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_contacts, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_free, cudaEventDisableTiming) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+        cudaEventCreateWithFlags(&h->ev_free, cudaEventDisableTiming) != cudaSuccess)
       return fail(PIBM_ECUDA);
-    h->side_grid = 4 * sms;  // a share of the GPU beside the coupling kernels
+    h->side_grid = 4 * s.sms;  // a share of the GPU beside the coupling kernels
     h->split = split;
     if (split == SPLIT_TILES) h->kernels_per_step += 1;
   }

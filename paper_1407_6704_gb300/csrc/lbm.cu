@@ -351,9 +351,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_sum_partials(const double* __re
 // 256 threads per CTA, or 64 where 256 would leave an SM fewer than four CTAs: the
 // cells of a small lattice then spread over every SM (its FP64 collision is bound by
 // the FP64 pipe of the SMs that have work).
-dim3 cell_block(const Geometry& g) {
-  constexpr long long SMS = 152;
-  const int t = g.ncell < 4 * SMS * 256 ? 64 : 256;
+dim3 cell_block(const State& s) {
+  const Geometry& g = s.geo;
+  const int t = g.ncell < 4LL * s.sms * 256 ? 64 : 256;
   const int bx = g.n[0] <= 32 ? 32 : (g.n[0] <= 64 || t == 64 ? 64 : 128);
   return dim3(bx, t / bx, 1);
 }
@@ -361,7 +361,7 @@ dim3 cell_block(const Geometry& g) {
 // Block shape of the fused collide-stream: the tuned one when set, else the default.
 dim3 collide_block(const State& s, bool pair) {
   if (s.cblk[0] > 0 && s.cblk[1] > 0) return dim3(s.cblk[0], s.cblk[1], 1);
-  return pair ? dim3(32, 8, 1) : cell_block(s.geo);
+  return pair ? dim3(32, 8, 1) : cell_block(s);
 }
 
 template <int Q, class St, typename FT>

@@ -21,12 +21,12 @@ namespace {
 // Warps per CTA of a kernel over `warps` warps of particles: 8, or fewer where CTAs of 8
 // would leave SMs idle (two CTAs per SM). Few particles in one CTA share the FP64 pipe of
 // one SM: 200 particles in 2D FP64 took 8.1 us to couple in one CTA, 6.9 in seven.
-unsigned warps_per_cta(long long warps) {
+unsigned warps_per_cta(const State& s, long long warps) {
   unsigned w = 8;
-  while (w > 1 && warps < 2LL * 152 * w) w /= 2;
+  while (w > 1 && warps < 2LL * s.sms * w) w /= 2;
   return w;
 }
-unsigned particle_threads(long long np) { return 32 * warps_per_cta((np + 31) / 32); }
+unsigned particle_threads(const State& s) { return 32 * warps_per_cta(s, (s.p.np + 31) / 32); }
 }  // namespace
 
 cudaError_t launch_bin(const State& s, cudaStream_t st, int* nk) {
@@ -35,7 +35,7 @@ cudaError_t launch_bin(const State& s, cudaStream_t st, int* nk) {
   cudaError_t e = cudaMemsetAsync(P.bin_cnt, 0, sizeof(unsigned) * (P.nbin + 1), st);
   if (e != cudaSuccess) return e;
   const double* X = P.X[s.cur];
-  const unsigned pt = particle_threads(P.np);
+  const unsigned pt = particle_threads(s);
   if (s.geo.d == 2)
     k_bin_key<2><<<blocks_for(P.np, pt), pt, 0, st>>>(X, P.np, s.geo, P.bm, P.cf[s.cur], P.key,
                                                         P.rank, P.bin_cnt, P.xr, P.cr);
@@ -82,7 +82,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
   using SC = typename std::conditional<IN_ORDER<St>, StoreF16, SA>::type;
   CoupleArgs A = couple_args(s);
   const long long ntiles = P.nbin / P.bm.tc;
-  const unsigned pt = IN_ORDER<St> ? 256 : particle_threads(P.np), pb = blocks_for(P.np, pt);
+  const unsigned pt = IN_ORDER<St> ? 256 : particle_threads(s), pb = blocks_for(P.np, pt);
   auto moments = [&](auto threads) {
     constexpr int TH = decltype(threads)::value;
     using Sh = MomentsShape<Q, St, TH>;
@@ -91,7 +91,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
             s.geo, P.bm, P.tbusy, P.tn, (const T*)s.f[s.cur], (R*)s.mom);
   };
   // small CTAs where the large ones would leave an SM fewer than four
-  if (s.geo.ncell < 4 * 152 * MomentsShape<Q, St>::CELLS)
+  if (s.geo.ncell < 4LL * s.sms * MomentsShape<Q, St>::CELLS)
     moments(std::integral_constant<int, 64>{});
   else
     moments(std::integral_constant<int, 256>{});
@@ -124,9 +124,9 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     // 16-bit storage keeps whole warps in CTAs of 256 threads (IN_ORDER).
     constexpr int PPW_FEW = W == 4 ? 8 : 16;
     const bool few =
-        P.np <= 4 * 152 * 32 && (COUPLE_BY_WARP<SC> || (D == 3 && !IN_ORDER<SC>));
+        P.np <= FEW_PARTICLES && (COUPLE_BY_WARP<SC> || (D == 3 && !IN_ORDER<SC>));
     auto couple = [&](auto kern, int ppw) {
-      const unsigned w = IN_ORDER<SC> ? COUPLE_WARPS : warps_per_cta((P.np + ppw - 1) / ppw);
+      const unsigned w = IN_ORDER<SC> ? COUPLE_WARPS : warps_per_cta(s, (P.np + ppw - 1) / ppw);
       static_assert(COUPLE_WARPS == 8, "warps_per_cta's largest");
       kern<<<blocks_for(P.np, w * ppw), w * 32, 0, st>>>(A);
     };
@@ -227,7 +227,7 @@ cudaError_t launch_contacts(const State& s, cudaStream_t st, int* nk) {
   // with DEM sub-cycling the contacts run inside the particle phase, per sub-step
   if (s.p.np == 0 || s.phy.substeps > 1) return cudaSuccess;
   CoupleArgs A = couple_args(s);
-  const unsigned pt = particle_threads(s.p.np);
+  const unsigned pt = particle_threads(s);
   const bool hs = contacts_half_shell(s);
   if (hs) {  // partner forces are added into the array: start from zero
     const cudaError_t e =

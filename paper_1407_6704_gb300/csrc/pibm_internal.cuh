@@ -420,6 +420,11 @@ struct Particles {
   unsigned* tn;     // [2] number of busy and free tiles
 };
 
+// The few-particle form of the coupling (particles.cu) serves up to this many: four warps
+// of 32 particles on each of 152 SMs. A number of its own and not the device's SM count:
+// the form decides the order of FP64 sums in 3D, which stays the same on any device.
+constexpr long long FEW_PARTICLES = 4LL * 152 * 32;
+
 // Tiles per CTA of the tile-list kernels.
 constexpr int TILE_BLOCK = 256;
 
@@ -432,6 +437,7 @@ struct State {
   Physics phy;
   int precision;
   int deterministic;
+  int sms;        // SMs of the device (CTA shapes)
   void* f[2];     // population buffers (post-collision of the last step), [q][pitch]
   void* F;        // force field [pitch][FieldStride], double (FP64) or float (FP32)
   void* mom;      // moment field [pitch][4] of the current state (cells near particles)
