@@ -123,8 +123,7 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     // count: an ensemble member equals the same simulation stepped alone bit for bit.
     // 16-bit storage keeps whole warps in CTAs of 256 threads (IN_ORDER).
     constexpr int PPW_FEW = W == 4 ? 8 : 16;
-    const bool few =
-        P.np <= FEW_PARTICLES && (COUPLE_BY_WARP<SC> || (D == 3 && !IN_ORDER<SC>));
+    constexpr bool FEW_FORM = COUPLE_BY_WARP<SC> || (D == 3 && !IN_ORDER<SC>);
     auto couple = [&](auto kern, int ppw) {
       const unsigned w = IN_ORDER<SC> ? COUPLE_WARPS : warps_per_cta(s, (P.np + ppw - 1) / ppw);
       static_assert(COUPLE_WARPS == 8, "warps_per_cta's largest");
@@ -132,8 +131,10 @@ cudaError_t couple_t(const State& s, cudaStream_t st, int* nk, cudaEvent_t befor
     };
     auto go = [&](auto lag, auto p64) {
       constexpr bool LAG = decltype(lag)::value, P64 = decltype(p64)::value;
-      if (few) couple(k_couple<QC, W, SC, FT, LAG, P64, PPW_FEW>, PPW_FEW);
-      else couple(k_couple<QC, W, SC, FT, LAG, P64, 32>, 32);
+      if constexpr (FEW_FORM) {
+        if (P.np <= FEW_PARTICLES) return couple(k_couple<QC, W, SC, FT, LAG, P64, PPW_FEW>, PPW_FEW);
+      }
+      couple(k_couple<QC, W, SC, FT, LAG, P64, 32>, 32);
     };
     using Yes = std::true_type;
     using No = std::false_type;
