@@ -1056,7 +1056,7 @@ int settling_gradient(const pibm_config* cfg_in, int64_t nsteps, int64_t K, void
   // kernels).
   StretchGraphs graphs;
   bool replayed = grads && nseg >= 4 && K <= 64 &&
-                  cudaStreamCreateWithFlags(&graphs.cap, cudaStreamNonBlocking) == cudaSuccess;
+                  make_capture_stream(&graphs.cap);
   // body(stream) enqueues stretch kind kd of K steps starting from parity key; the host
   // state it advances is s.cur (forward kinds) or io (reverse)
   auto stretch = [&](int kd, int key, auto&& body) -> cudaError_t {

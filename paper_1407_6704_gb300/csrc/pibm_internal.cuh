@@ -589,6 +589,19 @@ __device__ __forceinline__ void axis_taps_local(int c, float f, int n, int perio
   }
 }
 
+// A stream of its own to capture graphs on. False where none can be made, and then no
+// error stays behind: the caller goes on without graphs, and its next launch would report
+// it. The calls are parameters for the test.
+inline bool make_capture_stream(cudaStream_t* s,
+                                cudaError_t (*create)(cudaStream_t*, unsigned) =
+                                    cudaStreamCreateWithFlags,
+                                cudaError_t (*take_error)() = cudaGetLastError) {
+  if (create(s, cudaStreamNonBlocking) == cudaSuccess) return true;
+  (void)take_error();
+  *s = nullptr;
+  return false;
+}
+
 // ---------------------------------------------------------------------------
 // Launchers (defined in lbm.cu, particles.cu, reduce.cu)
 // ---------------------------------------------------------------------------
