@@ -57,7 +57,8 @@ __device__ __forceinline__ bool nonzero_bits(double v) { return __double_as_long
 __device__ __forceinline__ bool nonzero_bits(float v) { return __float_as_uint(v) != 0u; }
 
 // 1 / rho for the collision. rho is positive and near 1; one that is not raises the
-// health flag beside it.
+// health flag beside it. rho is 1 plus a rounded sum, so it is zero (flagged) or at
+// least 2^-53 in size: rcp_series never meets a subnormal one.
 __device__ __forceinline__ float inverse_density(float rho) { return 1.f / rho; }
 __device__ __forceinline__ double inverse_density(double rho) { return rcp_series(rho); }
 

@@ -118,8 +118,9 @@ struct StoreBF16 {
 // FP64 values without the FP64 pipe. It issues one warp instruction in 16 cycles
 // here, a conversion to or from FP64 as much as an addition, and it bounds the
 // FP64 kernels and most of the particle update; the same on the bit pattern is a
-// handful of integer instructions. Results are those of the plain operations for
-// every value (the rare ones take them).
+// handful of integer instructions. Results of widen, narrow, twice and from_index are
+// those of the plain operations for every value (the rare ones take them);
+// rcp_series holds where its comment says.
 // ---------------------------------------------------------------------------
 // FP32 -> FP64, exact.
 __device__ __forceinline__ double widen(float v) {
@@ -167,8 +168,10 @@ __device__ __forceinline__ double from_index(int c) {
 
 // 1 / d in FP64: the hardware's coarse reciprocal (PTX rcp.approx.ftz.f64, about 20
 // bits) and one third-order step of the series 1 / (1 - e) = 1 + e + e^2 + ...,
-// e = 1 - d r: three FP64 instructions for a result within a rounding of exact, about
-// half of what the division takes.
+// e = 1 - d r: three FP64 instructions for a result next to the division's at most, about
+// half of what the division takes. For d in 2^-1000 .. 2^1000; for zero, a subnormal
+// (flushed by the approximation), an infinity or NaN the result is not finite, where
+// the division's may be: callers that can meet those test for it and divide.
 __device__ __forceinline__ double rcp_series(double d) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
