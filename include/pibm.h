@@ -262,8 +262,8 @@ int pibm_profile_steps(pibm_t* h, int64_t nsteps, double* phase_ms);
  *   drho: [n_particles] dL/d(density ratio of each particle) (may be NULL),
  *   dx0:  [n_particles][d] dL/d(initial position) (may be NULL);
  * all host pointers. The forward run is the library's deterministic step; the
- * state is checkpointed every checkpoint_every steps and each stretch is
- * replayed for the reverse sweep, which needs device memory for
+ * state is checkpointed every checkpoint_every steps and each stretch but the last
+ * is replayed for the reverse sweep, which needs device memory for
  * (ceil(nsteps / checkpoint_every) + checkpoint_every) copies of the workspace of
  * pibm_workspace_bytes(cfg). The call allocates and frees that memory itself and
  * returns when done, on `stream` (a cudaStream_t, NULL = legacy default).
