@@ -393,6 +393,94 @@ struct DeviceGuard {
   }
 };
 
+// The launches and copies of pibm_read_fields, queued on the handle's stream.
+int queue_reads(pibm_t* h, unsigned mask, void* const* dst, int on_device) {
+  State& s = h->s;
+  const long long nc = s.geo.ncell, np = s.p.np;
+  const int d = s.geo.d, q = s.geo.q;
+  cudaStream_t st = h->stream;
+  // free between steps: the partner population buffer stages host reads
+  double* stage = (double*)s.f[1 - s.cur];
+  const size_t room = align_up((size_t)q * s.geo.pitch * pop_bytes(s.precision));
+  double* rho = mask & PIBM_FIELD_RHO ? (double*)dst[0] : nullptr;
+  double* mom = mask & PIBM_FIELD_J ? (double*)dst[1] : nullptr;
+  double* pop = mask & PIBM_FIELD_POP ? (double*)dst[2] : nullptr;
+  if (on_device) {
+    if (rho || mom || pop) CK(launch_read_state(s, rho, mom, pop, 0, pop ? q : 0, st));
+  } else {
+    const size_t bytes[PIBM_NFIELDS] = {sizeof(double) * nc, sizeof(double) * nc * d,
+                                        sizeof(double) * nc * q, sizeof(double) * d * np,
+                                        sizeof(double) * d * np};
+    for (int k = 0; k < PIBM_NFIELDS; ++k)
+      if (mask >> k & 1u) map_pages(dst[k], bytes[k]);
+    // as many planes per launch as the stage holds (rho, the d planes of j and the
+    // population planes, in this order); the copies follow their kernel on the
+    // stream, and the next launch follows them
+    const long long cap = (long long)(room / (sizeof(double) * nc));
+    int a = 0;
+    while (rho || mom || (pop && a < q)) {
+      long long used = 0;
+      double *srho = nullptr, *smom = nullptr, *spop = nullptr;
+      if (rho && used + 1 <= cap) {
+        srho = stage;
+        used += 1;
+      }
+      if (mom && used + d <= cap) {
+        smom = stage + used * nc;
+        used += d;
+      }
+      const int a0 = a;
+      if (pop && used < cap) {
+        spop = stage + used * nc;
+        a = (int)std::min<long long>(q, a0 + (cap - used));
+      }
+      if (!srho && !smom && !spop) return PIBM_EINTERNAL;  // the stage holds j in every mode
+      CK(launch_read_state(s, srho, smom, spop, a0, a, st));
+      const size_t plane = sizeof(double) * nc;
+      if (srho) CK(cudaMemcpyAsync(rho, srho, plane, cudaMemcpyDeviceToHost, st));
+      if (smom) CK(cudaMemcpyAsync(mom, smom, plane * d, cudaMemcpyDeviceToHost, st));
+      if (a > a0)
+        CK(cudaMemcpyAsync(pop + (size_t)a0 * nc, spop, plane * (a - a0), cudaMemcpyDeviceToHost,
+                           st));
+      if (srho) rho = nullptr;
+      if (smom) mom = nullptr;
+    }
+  }
+  double* ox = mask & PIBM_FIELD_X && np > 0 ? (double*)dst[3] : nullptr;
+  double* ou = mask & PIBM_FIELD_U && np > 0 ? (double*)dst[4] : nullptr;
+  const size_t vb = sizeof(double) * d * np;
+  if (on_device) {
+    CK(launch_interleave(s, ox, ou, st));
+  } else if (2 * vb <= room) {
+    // storage order -> user order on the device, then one copy per field into the
+    // caller's array
+    double *sx = stage, *su = stage + (size_t)d * np;
+    CK(launch_interleave(s, ox ? sx : nullptr, ou ? su : nullptr, st));
+    if (ox) CK(cudaMemcpyAsync(ox, sx, vb, cudaMemcpyDeviceToHost, st));
+    if (ou) CK(cudaMemcpyAsync(ou, su, vb, cudaMemcpyDeviceToHost, st));
+  } else {
+    // a lattice too small to stage the particles: storage order -> user order
+    // on the host
+    std::vector<double> soa((size_t)d * np);
+    std::vector<unsigned> pid((size_t)np);
+    for (int f = 0; f < 2; ++f) {
+      double* o = f == 0 ? ox : ou;
+      if (!o) continue;
+      const double* src = f == 0 ? s.p.X[s.cur] : s.p.U[s.cur];
+      CK(cudaMemcpyAsync(soa.data(), src, vb, cudaMemcpyDeviceToHost, st));
+      CK(cudaMemcpyAsync(pid.data(), s.p.pid[s.cur], sizeof(unsigned) * np,
+                         cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      for (long long i = 0; i < np; ++i) {
+        const unsigned p = pid[(size_t)i];
+        if (p >= (unsigned long long)np) return PIBM_EINTERNAL;
+        for (int k = 0; k < d; ++k) o[(size_t)p * d + k] = soa[(size_t)k * np + i];
+      }
+    }
+  }
+  return PIBM_OK;
+}
+
 }  // namespace
 
 namespace pibm {
@@ -758,88 +846,10 @@ int pibm_read_fields(pibm_t* h, unsigned mask, void* const* dst, int on_device) 
   for (int k = 0; k < PIBM_NFIELDS; ++k)
     if ((mask >> k & 1u) && !dst[k]) return PIBM_EINVAL;
   DeviceGuard guard(h->device);
-  State& s = h->s;
-  const long long nc = s.geo.ncell, np = s.p.np;
-  const int d = s.geo.d, q = s.geo.q;
-  cudaStream_t st = h->stream;
-  // free between steps: the partner population buffer stages host reads
-  double* stage = (double*)s.f[1 - s.cur];
-  const size_t room = align_up((size_t)q * s.geo.pitch * pop_bytes(s.precision));
-  double* rho = mask & PIBM_FIELD_RHO ? (double*)dst[0] : nullptr;
-  double* mom = mask & PIBM_FIELD_J ? (double*)dst[1] : nullptr;
-  double* pop = mask & PIBM_FIELD_POP ? (double*)dst[2] : nullptr;
-  if (on_device) {
-    if (rho || mom || pop) CK(launch_read_state(s, rho, mom, pop, 0, pop ? q : 0, st));
-  } else {
-    const size_t bytes[PIBM_NFIELDS] = {sizeof(double) * nc, sizeof(double) * nc * d,
-                                        sizeof(double) * nc * q, sizeof(double) * d * np,
-                                        sizeof(double) * d * np};
-    for (int k = 0; k < PIBM_NFIELDS; ++k)
-      if (mask >> k & 1u) map_pages(dst[k], bytes[k]);
-    // as many planes per launch as the stage holds (rho, the d planes of j and the
-    // population planes, in this order); the copies follow their kernel on the
-    // stream, and the next launch follows them
-    const long long cap = (long long)(room / (sizeof(double) * nc));
-    int a = 0;
-    while (rho || mom || (pop && a < q)) {
-      long long used = 0;
-      double *srho = nullptr, *smom = nullptr, *spop = nullptr;
-      if (rho && used + 1 <= cap) {
-        srho = stage;
-        used += 1;
-      }
-      if (mom && used + d <= cap) {
-        smom = stage + used * nc;
-        used += d;
-      }
-      const int a0 = a;
-      if (pop && used < cap) {
-        spop = stage + used * nc;
-        a = (int)std::min<long long>(q, a0 + (cap - used));
-      }
-      if (!srho && !smom && !spop) return PIBM_EINTERNAL;  // the stage holds j in every mode
-      CK(launch_read_state(s, srho, smom, spop, a0, a, st));
-      const size_t plane = sizeof(double) * nc;
-      if (srho) CK(cudaMemcpyAsync(rho, srho, plane, cudaMemcpyDeviceToHost, st));
-      if (smom) CK(cudaMemcpyAsync(mom, smom, plane * d, cudaMemcpyDeviceToHost, st));
-      if (a > a0)
-        CK(cudaMemcpyAsync(pop + (size_t)a0 * nc, spop, plane * (a - a0), cudaMemcpyDeviceToHost,
-                           st));
-      if (srho) rho = nullptr;
-      if (smom) mom = nullptr;
-    }
-  }
-  double* ox = mask & PIBM_FIELD_X && np > 0 ? (double*)dst[3] : nullptr;
-  double* ou = mask & PIBM_FIELD_U && np > 0 ? (double*)dst[4] : nullptr;
-  const size_t vb = sizeof(double) * d * np;
-  if (on_device) {
-    CK(launch_interleave(s, ox, ou, st));
-  } else if (2 * vb <= room) {
-    // storage order -> user order on the device, then one copy per field into the
-    // caller's array
-    double *sx = stage, *su = stage + (size_t)d * np;
-    CK(launch_interleave(s, ox ? sx : nullptr, ou ? su : nullptr, st));
-    if (ox) CK(cudaMemcpyAsync(ox, sx, vb, cudaMemcpyDeviceToHost, st));
-    if (ou) CK(cudaMemcpyAsync(ou, su, vb, cudaMemcpyDeviceToHost, st));
-  } else {
-    // a lattice too small to stage the particles: storage order -> user order
-    // on the host
-    std::vector<double> soa((size_t)d * np);
-    std::vector<unsigned> pid((size_t)np);
-    for (int f = 0; f < 2; ++f) {
-      double* o = f == 0 ? ox : ou;
-      if (!o) continue;
-      const double* src = f == 0 ? s.p.X[s.cur] : s.p.U[s.cur];
-      CK(cudaMemcpyAsync(soa.data(), src, vb, cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(pid.data(), s.p.pid[s.cur], sizeof(unsigned) * np,
-                         cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      for (long long i = 0; i < np; ++i) {
-        const unsigned p = pid[(size_t)i];
-        if (p >= (unsigned long long)np) return PIBM_EINTERNAL;
-        for (int k = 0; k < d; ++k) o[(size_t)p * d + k] = soa[(size_t)k * np + i];
-      }
-    }
+  const int rc = queue_reads(h, mask, dst, on_device);
+  if (rc != PIBM_OK) {  // copies into the caller's pinned arrays may be in flight
+    cudaStreamSynchronize(h->stream);
+    return rc;
   }
   return health(h);
 }
